@@ -46,6 +46,8 @@ struct vmc_ctx {
   int n_work = 0;
   int *d_work_ctr = nullptr;
   size_t smem_sample = 0, smem_init = 0;
+  int n_max = 1;              // largest N of the systems
+  int init_form = VMC_INIT_BLOCKED;   // how from-scratch inverses are formed
   int grid_sample = 0;
   long long n_launch = 0;
   double *d_scalar = nullptr;
@@ -60,6 +62,7 @@ struct vmc_ctx {
   cudaEvent_t fork_ev = nullptr, join_ev[NPOOL] = {};
   size_t smem_cap = 0;        // dynamic shared-memory limit set on the sweep kernels
   size_t smem_proj = 0;       // projected sweep kernel (vmc_set_projection)
+  size_t smem_build = 0;      // from-scratch inverses of the projected state
   int grid_proj = 0;
   void *corr_buf = nullptr;   // vmc_measure_corr scratch (grown on demand)
   size_t corr_bytes = 0;
@@ -352,10 +355,11 @@ int periodic_rebuild(vmc_ctx *c) {
   TimedRegion tr(c, 1);
   if (projected(c))
     CKC(vmc_launch_proj_build(c->d_sys, c->d_work, c->n_work, c->sys[0].dev.n_ops, c->precision,
-                              1, c->recompute_every, c->smem_init, c->st, &c->n_launch));
+                              c->n_max, 1, c->recompute_every, c->smem_build, c->st, &c->n_launch));
   else
-    CKC(vmc_launch_init(c->d_sys, c->d_work, c->n_work, c->d_work_ctr + 1, c->precision, 1,
-                        c->recompute_every, c->smem_init, c->st, &c->n_launch));
+    CKC(vmc_launch_init(c->d_sys, c->d_work, c->n_work, c->d_work_ctr + 1, c->precision,
+                        c->init_form, c->n_max, 1, c->recompute_every, c->smem_init, c->st,
+                        &c->n_launch));
   c->rebuild_pending = false;
   return VMC_OK;
 }
@@ -379,11 +383,10 @@ int ensure_init(vmc_ctx *c, bool redraw_illcond = false) {
     TimedRegion tr(c, 1);
     if (c->n_sys == 1 && c->sys[0].dev.n_ops > 0)
       CKC(vmc_launch_proj_build(c->d_sys, c->d_work, c->n_work, c->sys[0].dev.n_ops, c->precision,
-                                0, 0, c->smem_init, c->st, &c->n_launch));
+                                c->n_max, 0, 0, c->smem_build, c->st, &c->n_launch));
     else
-      CKC(vmc_launch_init(c->d_sys, c->d_work, c->n_work, c->d_work_ctr + 1, c->precision, 0, 0,
-                          c->smem_init, c->st,
-                          &c->n_launch));
+      CKC(vmc_launch_init(c->d_sys, c->d_work, c->n_work, c->d_work_ctr + 1, c->precision,
+                          c->init_form, c->n_max, 0, 0, c->smem_init, c->st, &c->n_launch));
   }
   int bad = 0;
   for (auto &s : c->sys) {
@@ -546,7 +549,7 @@ int create_impl(vmc_ctx **out, int n_sys, const vmc_model *models, const int32_t
   const int esize = o->precision == VMC_FP64 ? 8 : 4;
   int rc = VMC_OK;
   size_t smem64 = 0, smem32 = 0;
-  int maxN = 1;
+  bool exchange = false;      // some system has exchange terms
   auto fail = [&](int e) {
     ctx_free(c);
     delete c;
@@ -569,7 +572,7 @@ int create_impl(vmc_ctx **out, int n_sys, const vmc_model *models, const int32_t
     s.W = o->n_walkers;
     s.max_samples = o->max_samples;
     s.p_exchange = m.local_spin ? 1.0 : (pex ? pex[si] : 0.0);
-    maxN = std::max(maxN, s.N);
+    c->n_max = std::max(c->n_max, s.N);
     SysDev &d = s.dev;
     d.Ns = s.Ns;
     d.Ne = s.Ne;
@@ -725,7 +728,7 @@ int create_impl(vmc_ctx **out, int n_sys, const vmc_model *models, const int32_t
     smem64 = std::max(smem64, vmc_walker_smem(0, s.N, s.Ns, s.Np, H, 0, &acc_len, 0));
     smem32 = std::max(smem32, vmc_walker_smem(1, s.N, s.Ns, s.Np, H, 0, &acc_len, 1));
     d.acc_len = acc_len;
-    c->smem_init = std::max(c->smem_init, vmc_init_smem(s.N, s.Ns));
+    exchange |= m.n_J > 0;
     if (vmc_launch_expand(&d, c->st, &c->n_launch) != cudaSuccess) return fail(VMC_ECUDA);
     // seeded random placement
     std::vector<int32_t> ele(W * s.Ne);
@@ -738,6 +741,10 @@ int create_impl(vmc_ctx **out, int n_sys, const vmc_model *models, const int32_t
       return fail(VMC_ECUDA);
   }
   c->smem_sample = (c->precision == VMC_FP64) ? smem64 : smem32;
+  c->init_form = vmc_init_form(c->precision == VMC_FP64 ? 0 : 1,
+                               o->rebuild == VMC_REBUILD_DOUBLE_FLOAT, exchange, c->n_max);
+  for (const SysHost &s : c->sys)
+    c->smem_init = std::max(c->smem_init, vmc_init_smem(s.N, s.Ns, c->init_form));
   {
     // The sweep kernels may use up to the device's opt-in limit (less the
     // static part): delayed updates enlarge the walker's shared state.
@@ -1543,7 +1550,8 @@ int vmc_set_projection(vmc_ctx *c, int32_t n_ops, const int32_t *perm, const int
   if ((rc = dalloc(c, &d.ppi, sizeof(double) * W * n_ops))) return rc;
   if ((rc = dalloc(c, &d.plog, sizeof(double) * W * n_ops))) return rc;
   if ((rc = dalloc(c, &d.psign, sizeof(int) * W * n_ops))) return rc;
-  CKC(vmc_proj_set_smem(smem, c->smem_init));
+  c->smem_build = vmc_proj_build_smem(c->precision == VMC_FP64 ? 0 : 1, s.N);
+  CKC(vmc_proj_set_smem(smem, c->smem_build));
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int occ = std::max(1, vmc_proj_occupancy(c->precision, smem));

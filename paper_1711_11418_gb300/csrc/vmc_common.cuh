@@ -116,9 +116,14 @@ __device__ __forceinline__ int vmc_mulhi(uint32_t r, int n) {
 // ---- launch wrappers (defined in vmc_walker.cu / vmc_sr.cu) ----
 // All return cudaError_t from the launch; they count launches in *n_launch.
 cudaError_t vmc_launch_expand(const SysDev *h_sys, cudaStream_t st, long long *n_launch);
+// How the from-scratch inverses are formed: FP64 by panels, FP64 step by step
+// (small N, and the mixed form of models with exchange terms, where last bits
+// show in a trajectory; vmc_gj.cuh), double-float (the mixed form's opt-in).
+enum { VMC_INIT_BLOCKED = 0, VMC_INIT_STEPS = 1, VMC_INIT_DF = 2 };
+int vmc_init_form(int precision, int df, int exchange, int n_max);
 cudaError_t vmc_launch_init(const SysDev *d_sys, const int2 *d_work, int n_work, int *d_ctr,
-                            int precision, int only_due, int due_threshold, size_t smem,
-                            cudaStream_t st, long long *nl);
+                            int precision, int form, int n_max, int only_due, int due_threshold,
+                            size_t smem, cudaStream_t st, long long *nl);
 cudaError_t vmc_launch_sample(const SysDev *d_sys, const int2 *d_work, int n_work,
                               int *d_work_ctr, int precision, uint64_t seed,
                               int n_first, int n_samples, int sweeps_between,
@@ -144,7 +149,7 @@ cudaError_t vmc_launch_corr_reduce(const double *part, int n_part, const int *cn
 // M^-1 in shared memory as well (the pair-correlation kernel does not).
 size_t vmc_walker_smem(int precision, int N, int Ns, int Np, int H, int kd, int *acc_len,
                        int with_lo);
-size_t vmc_init_smem(int N, int Ns);
+size_t vmc_init_smem(int N, int Ns, int form);
 int vmc_sample_occupancy(int precision, size_t smem);
 // the mixed form's 168-register sweep variant (vmc_sweep3.cu)
 int vmc_sample_occupancy_v3(size_t smem);
@@ -158,11 +163,12 @@ cudaError_t vmc_walker_set_smem_limits(size_t smem_sample64, size_t smem_sample3
 
 // Projected wave function (vmc_proj.cu)
 size_t vmc_proj_smem(int precision, int N, int Ns, int n_ops);
+size_t vmc_proj_build_smem(int precision, int N);
 int vmc_proj_occupancy(int precision, size_t smem);
 cudaError_t vmc_proj_set_smem(size_t s_sample, size_t s_build);
 cudaError_t vmc_launch_proj_build(const SysDev *d_sys, const int2 *d_work, int n_work, int n_ops,
-                                  int precision, int only_due, int due_threshold, size_t smem,
-                                  cudaStream_t st, long long *n_launch);
+                                  int precision, int n_max, int only_due, int due_threshold,
+                                  size_t smem, cudaStream_t st, long long *n_launch);
 cudaError_t vmc_launch_proj_sample(const SysDev *d_sys, const int2 *d_work, int n_work,
                                    int *d_work_ctr, int precision, uint64_t seed, int n_first,
                                    int n_samples, int sweeps_between, int sample_base, int grid,

@@ -1,17 +1,453 @@
-// From-scratch inverse of one walker's M: FP64 Gauss-Jordan elimination with
-// partial pivoting in shared memory (mVMC paper, Sec. 3.2.1: the Pfaffian of
-// the anti-parallel pair product is det M up to a sign, Pf^2 = det X), with
-// log|det M| and its sign.  Shared by the translation units of the walker
-// kernels (the plain walker and the projected one).
+// From-scratch inverse of one walker's M in FP64: blocked Gauss-Jordan
+// elimination with partial pivoting in shared memory (mVMC paper, Sec. 3.2.1:
+// the Pfaffian of the anti-parallel pair product is det M up to a sign,
+// Pf^2 = det X), with log|det M| and its sign.  Shared by the translation
+// units of the walker kernels (the plain walker and the projected one).
+//
+// In place on M padded to Npad rows and columns (a multiple of GB, identity
+// in the padding), GB columns (a panel) at a time:
+//   panel   one thread per row holds its GB entries in registers and takes
+//           the GB elimination steps in FP64.  Rows are not moved: the row
+//           that is the pivot of step k keeps its place (perm[k] = row).  The
+//           panel then holds T (Npad x GB), the effect of its steps on every
+//           other column;
+//   update  A <- A_masked + T R for the columns outside the panel, R the GB
+//           pivot rows before the panel and A_masked the rest (pivot rows 0).
+// The update is a contraction over GB = 16 and nearly all of the
+// multiply-adds, so it runs on the tensor cores, in fixed point: each row of
+// T and each column of R becomes 56-bit integers (one exponent per row and
+// column, after a power of two per pivot row that evens out R's rows), cut
+// into seven signed 8-bit digits, which BF16 holds; the products of digits
+// s + u = d are summed by mma.sync m16n8k16 in FP32 without rounding
+// (integers below 2^23), d = 0..7; the eight sums make one integer, rounded
+// once to FP64 and added to A.  (Splitting operands so that sums of products
+// are free of error: Ozaki, Ogita, Oishi, Rump, Numer. Algorithms 59, 95,
+// 2012.)  What is left out is about 2^-56 of (row maximum of T) x (column
+// maximum of R), once per panel, where the elimination step by step rounds
+// every entry once per step.
+//
+// What bounds it: the FP64 pipe (2 multiply-adds per clock and SM), which has
+// the panels' N^2 GB multiply-adds and the update's N^3 / GB additions left
+// of N^3, and the pivot chain of the panels.  4096 walkers, N = 112: 5.1 ms
+// against 13.65 step by step; N = 128: 9.0 against 26.7; N = 64: 1.8 against
+// 3.2.  mma.sync and not tcgen05: a tile's products are consumed at once
+// by the warp that made them, eight 112 x 112 accumulators do not fit tensor
+// memory, and two walkers share an SM so that one's panel chain runs under
+// the other's update.
 #pragma once
 
 #include "vmc_common.cuh"
 
 namespace vmc_gj {
 
-constexpr int NT = VMC_NT;
-constexpr int NWARP = NT / 32;
+constexpr int GB = 16;               // panel width: K of one mma.sync m16n8k16
+constexpr int NDIG = 7;              // 8-bit digits of an operand
+constexpr int CT = 4;                // column tiles (of 8) whose digits are staged at a time
+constexpr int MAX_THREADS = 2 * VMC_MAX_N;
+constexpr int NOEXP = -(1 << 20);    // exponent of a group of zeros
 
+__host__ __device__ inline int gj_pad(int N) { return (N + GB - 1) / GB * GB; }
+// A warp per 16 rows for the update (a thread per row for the panel).
+__host__ __device__ inline int gj_threads(int N) {
+  const int t = (2 * gj_pad(N) + 31) / 32 * 32;
+  return t < 64 ? 64 : t;
+}
+// Up to this N the step-by-step form below is taken: its kernels need 48
+// registers a thread against 126, and the work per site around so small an
+// elimination wants the CTAs (4096 walkers, Ns = 256: N = 8 1.03 ms against
+// 1.20, N = 24 1.08 against 1.20; N = 32 1.20 against 1.16, N = 48 1.85
+// against 1.47).
+constexpr int GJ_STEPS_MAX_N = 24;
+// Shared memory (bytes): the matrix, then the staged digits of R (free after
+// the elimination).
+__host__ __device__ inline size_t gj_matrix_bytes(int N) {
+  return (size_t)gj_pad(N) * gj_pad(N) * sizeof(double);
+}
+constexpr size_t GJ_STAGE_BYTES = (size_t)NDIG * CT * 8 * 8 * sizeof(uint32_t);
+
+// Entry (i, c) of the matrix: rows of Npad doubles, the 64-byte halves of
+// each 128-byte group swapped in odd rows, so that the 16-byte accesses of an
+// accumulator tile (two rows per eight lanes) touch every bank once.
+__host__ __device__ inline int gj_at(int i, int c, int ld) { return i * ld + (c ^ ((i & 1) << 3)); }
+
+struct GJShared {
+  alignas(16) double cand[2][4][GB];   // candidate pivot row of each panel warp, by step parity
+  unsigned long long ckey[2][4];
+  double cinv[2][4];
+  int crow[2][4];
+  int perm[VMC_MAX_N];         // row that is the pivot of step k
+  int step[VMC_MAX_N];         // step of which row i is the pivot
+  int sig[GB];                 // power of two taken out of each pivot row
+  int rexp[CT * 8];            // exponent of each staged column of R
+  double val[4], pminw[4], amax[4];
+  int neg[4];
+  int bad, nonfinite;
+  int sign;
+  double logdet, pmin, pmax;   // log|det M|, smallest / largest |pivot|
+};
+
+// ---- 56-bit fixed point in digits -------------------------------------------
+// Biased exponent of x (0: zero or subnormal, taken as zero).
+__device__ __forceinline__ int gj_expo(double x) {
+  return (int)(((unsigned)__double2hiint(x) >> 20) & 0x7ffu);
+}
+
+// x 2^(55 - (e - 1022)) rounded to an integer, |q| <= 2^55, for |x| < 2^(e - 1022),
+// plus 128 in each of the six lower bytes: digit 0 (weight 2^48) is the value of
+// the bits from 48 up, digit s = 1..6 (weight 2^(48 - 8 s)) byte 6 - s less 128.
+__device__ __forceinline__ long long gj_fixed(double x, int e) {
+  const long long b = __double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 0x7ff);
+  const int d = min(max(e - ex, 0), 56);
+  long long m = ((b & 0x000fffffffffffffll) | 0x0010000000000000ll) << 2;   // 55 bits
+  m = (m + ((1ll << d) >> 1)) >> d;
+  if (ex == 0) m = 0;
+  return (b < 0 ? -m : m) + 0x0000808080808080ll;
+}
+
+// Digit s of v as a float (an integer in [-128, 128], exact in BF16): the byte
+// placed under the exponent of 2^23, less 2^23 + 128.
+__device__ __forceinline__ float gj_digit(long long v, int s) {
+  const unsigned hi = (unsigned)(v >> 32), lo = (unsigned)v;
+  if (s == 0) return __int_as_float(0x4B000200 + ((int)hi >> 16)) - 8389120.0f;
+  const unsigned w = s <= 2 ? hi : lo;
+  const unsigned k = s <= 2 ? 2 - s : 6 - s;
+  return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440u + k)) - 8388736.0f;
+}
+// Digits s of two values as a BF16 pair (exact: the upper halves).
+__device__ __forceinline__ uint32_t gj_pair(long long v0, long long v1, int s) {
+  return __byte_perm(__float_as_uint(gj_digit(v0, s)), __float_as_uint(gj_digit(v1, s)), 0x7632u);
+}
+
+// V 2^x as a double (to nearest, ties away from zero; |V| < 2^62).
+__device__ __forceinline__ double gj_scaled(long long V, int x) {
+  const unsigned long long s = (unsigned long long)V & 0x8000000000000000ull;
+  unsigned long long u = (unsigned long long)(V < 0 ? -V : V);
+  const int lz = __clzll((long long)u);
+  const int e = 1023 + 63 - lz + x;
+  // bit 63 set, half of the last of 53 places added (a carry out of the top
+  // reaches the exponent), the leading bit added to the exponent field
+  u = ((u << (lz & 63)) + 0x400ull);
+  const unsigned long long m = (u >> 11) | (u < 0x400ull ? 0x0020000000000000ull : 0ull);
+  unsigned long long b = s | (((unsigned long long)(unsigned)(e - 1) << 52) + m);
+  if (V == 0 || e <= 0) b = 0;
+  if (V != 0 && e >= 2046) b = s | 0x7ff0000000000000ull;
+  return __longlong_as_double((long long)b);
+}
+
+// The accumulators start at 1.5 x 2^23, so that their bits hold the integers.
+constexpr float GJ_MAGIC = 12582912.0f;
+constexpr int GJ_MAGIC_BITS = 0x4B400000;
+
+// Sum of the digit products (bits of the accumulators d = 0..7) in units of
+// 2^(E + F - 54) with T < 2^E, R < 2^F; d = 6 and 7 round into d = 5.
+__device__ __forceinline__ long long gj_combine(const float (&a)[8][4], int q) {
+  int n[8];
+#pragma unroll
+  for (int d = 0; d < 8; ++d) n[d] = __float_as_int(a[d][q]) - GJ_MAGIC_BITS;
+  const int p0 = n[0] * 256 + n[1], p1 = n[2] * 256 + n[3];
+  const int p2 = n[4] * 256 + n[5] + ((n[6] * 256 + n[7] + 32768) >> 16);
+  return (long long)p0 * 4294967296ll + (long long)p1 * 65536ll + (long long)p2;
+}
+
+__device__ __forceinline__ void gj_mma(float (&c)[4], const uint32_t (&a)[4], uint32_t b0,
+                                       uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// 1 / x by Newton's iteration from the hardware's 20-bit approximation; very
+// large and small x by the division.
+__device__ __forceinline__ double gj_recip(double x) {
+  const int e = gj_expo(x);
+  if (e < 64 || e > 1982) return 1.0 / x;
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  y = fma(fma(-x, y, 1.0), y, y);
+  return fma(fma(-x, y, 1.0), y, y);
+}
+
+// GB elimination steps on the panel of columns k0 .. k0 + GB - 1; threads
+// tid < 32 ceil(Npad / 32), row tid each.  `mine` is the step of which this
+// thread's row is the pivot (-1: none yet), `piv` that pivot.  Per step each
+// warp's candidate (largest |a| among rows not yet used, ties to the lowest
+// row) is published with its row and reciprocal, one barrier, and every
+// thread takes the best of them.
+__device__ __forceinline__ void gj_panel(double *A, int ld, int Npad, int k0, int &mine, double &piv,
+                                         GJShared &g) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nw = (Npad + 31) >> 5;
+  const bool row_ok = tid < Npad;
+  double r[GB];
+#pragma unroll
+  for (int j = 0; j < GB; j += 2) {
+    double2 v = make_double2(0.0, 0.0);
+    if (row_ok) v = *reinterpret_cast<const double2 *>(A + gj_at(tid, k0 + j, ld));
+    r[j] = v.x;
+    r[j + 1] = v.y;
+  }
+#pragma unroll
+  for (int k = 0; k < GB; ++k) {
+    const int buf = k & 1;
+    unsigned hi = (unsigned)__double2hiint(r[k]) & 0x7fffffffu, lo = (unsigned)__double2loint(r[k]);
+    const bool use = row_ok && mine < 0 && !(hi > 0x7ff00000u || (hi == 0x7ff00000u && lo != 0u));
+    if (!use) hi = lo = 0u;
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+    const unsigned bal = __ballot_sync(0xffffffffu, use && hi == mh && lo == ml);
+    if (bal ? lane == __ffs(bal) - 1 : lane == 0) {
+      g.ckey[buf][warp] = bal ? ((unsigned long long)mh << 32) | ml : 0ull;
+      g.crow[buf][warp] = tid;
+      g.cinv[buf][warp] = gj_recip(r[k]);
+#pragma unroll
+      for (int j = 0; j < GB; j += 2)
+        *reinterpret_cast<double2 *>(&g.cand[buf][warp][j]) = make_double2(r[j], r[j + 1]);
+    }
+    if (nw > 1)
+      asm volatile("bar.sync 1, %0;" ::"r"(nw * 32) : "memory");
+    else
+      __syncwarp();
+    int wb = 0;
+    unsigned long long bk = g.ckey[buf][0];
+    for (int q = 1; q < nw; ++q) {
+      const unsigned long long kq = g.ckey[buf][q];
+      if (kq > bk) {
+        bk = kq;
+        wb = q;
+      }
+    }
+    if (bk == 0ull) {   // no finite non-zero entry left: singular (every thread agrees)
+      if (tid == 0) g.bad = 1;
+      return;
+    }
+    const int p = g.crow[buf][wb];
+    const double ip = g.cinv[buf][wb];
+    const bool is = tid == p;
+    if (is) {
+      mine = k0 + k;
+      piv = r[k];
+      g.perm[k0 + k] = p;
+#pragma unroll
+      for (int j = 0; j < GB; ++j) r[j] = 0.0;
+    }
+    const double m = is ? ip : -(r[k] * ip);
+#pragma unroll
+    for (int j = 0; j < GB; j += 2) {
+      const double2 v = *reinterpret_cast<const double2 *>(&g.cand[buf][wb][j]);
+      if (j != k) r[j] = fma(m, v.x, r[j]);
+      if (j + 1 != k) r[j + 1] = fma(m, v.y, r[j + 1]);
+    }
+    r[k] = m;
+  }
+  if (row_ok) {
+    g.step[tid] = mine;
+#pragma unroll
+    for (int j = 0; j < GB; j += 2)
+      *reinterpret_cast<double2 *>(A + gj_at(tid, k0 + j, ld)) = make_double2(r[j], r[j + 1]);
+  }
+}
+
+// In place on the padded matrix A (gj_at); blockDim.x >= gj_threads(N).  On
+// return entry (k, c) of the inverse is A[perm[k]][step[c]] (gj_inverse_at).
+__device__ __forceinline__ void gj_invert(double *A, uint32_t *stage, int N, GJShared &g) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int Npad = gj_pad(N), ld = Npad, nwarps = blockDim.x >> 5;
+  const int np = (Npad + 31) >> 5;      // panel warps
+  const int nrb = Npad / 16;            // row blocks of the update, one per warp
+  const int gr = lane >> 2, gt = lane & 3;
+  int mine = -1;
+  double piv = 1.0;
+  if (tid == 0) g.bad = g.nonfinite = 0;
+  __syncthreads();
+  for (int k0 = 0; k0 < Npad; k0 += GB) {
+    if (warp < np) gj_panel(A, ld, Npad, k0, mine, piv, g);
+    __syncthreads();
+    if (g.bad) return;   // uniform
+    const int ntile = Npad / 8 - 2;
+    if (ntile == 0) break;
+    // the power of two of each pivot row outside the panel
+    for (int l = warp; l < GB; l += nwarps) {
+      const int p = g.perm[k0 + l];
+      int h = 0;
+      for (int c = lane; c < Npad; c += 32)
+        if (c < k0 || c >= k0 + GB) h = max(h, gj_expo(A[gj_at(p, c, ld)]));
+      h = __reduce_max_sync(0xffffffffu, h);
+      if (lane == 0) g.sig[l] = h ? h - 1023 : 0;
+    }
+    __syncthreads();
+    // this warp's 16 rows of T as digits: the A operands of the update
+    uint32_t a[NDIG][4];
+    int ea = NOEXP, eb = NOEXP;
+    const int ra = warp * 16 + gr, rb = ra + 8;
+    bool pa = false, pb = false;
+    if (warp < nrb) {
+      double x[2][4];
+      int sg[4];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const double2 u = *reinterpret_cast<const double2 *>(A + gj_at(ra, k0 + 2 * gt + 8 * h, ld));
+        const double2 v = *reinterpret_cast<const double2 *>(A + gj_at(rb, k0 + 2 * gt + 8 * h, ld));
+        x[0][2 * h] = u.x;
+        x[0][2 * h + 1] = u.y;
+        x[1][2 * h] = v.x;
+        x[1][2 * h + 1] = v.y;
+        sg[2 * h] = g.sig[2 * gt + 8 * h];
+        sg[2 * h + 1] = g.sig[2 * gt + 8 * h + 1];
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int e0 = gj_expo(x[0][q]), e1 = gj_expo(x[1][q]);
+        if (e0) ea = max(ea, e0 + sg[q]);
+        if (e1) eb = max(eb, e1 + sg[q]);
+        if (e0 == 0x7ff || e1 == 0x7ff) g.nonfinite = 1;
+      }
+      ea = max(ea, __shfl_xor_sync(0xffffffffu, ea, 1));
+      eb = max(eb, __shfl_xor_sync(0xffffffffu, eb, 1));
+      ea = max(ea, __shfl_xor_sync(0xffffffffu, ea, 2));
+      eb = max(eb, __shfl_xor_sync(0xffffffffu, eb, 2));
+      long long q0[4], q1[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        q0[q] = gj_fixed(x[0][q], ea - sg[q]);
+        q1[q] = gj_fixed(x[1][q], eb - sg[q]);
+      }
+#pragma unroll
+      for (int s = 0; s < NDIG; ++s) {
+        a[s][0] = gj_pair(q0[0], q0[1], s);
+        a[s][1] = gj_pair(q1[0], q1[1], s);
+        a[s][2] = gj_pair(q0[2], q0[3], s);
+        a[s][3] = gj_pair(q1[2], q1[3], s);
+      }
+      pa = g.step[ra] >= k0;
+      pb = g.step[rb] >= k0;
+    }
+    for (int c0 = 0; c0 < ntile; c0 += CT) {
+      const int nt = min(CT, ntile - c0);
+      // digits of the pivot rows' entries in these columns, four threads to a
+      // column: words (k pair t, k pair t + 4) of digit s of column j at
+      // stage[(32 s + j) 8 + 2 t], as the B operands read them
+      for (int q = tid; q < nt * 32; q += blockDim.x) {
+        const int j = q >> 2, t = q & 3;
+        const int tile = c0 + (j >> 3);
+        const int c = (tile < k0 / 8 ? tile : tile + 2) * 8 + (j & 7);
+        double x[4];
+        int sg[4], e = NOEXP;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int l = 2 * t + (u & 1) + 8 * (u >> 1);
+          x[u] = A[gj_at(g.perm[k0 + l], c, ld)];
+          sg[u] = g.sig[l];
+          const int ex = gj_expo(x[u]);
+          if (ex) e = max(e, ex - sg[u]);
+          if (ex == 0x7ff) g.nonfinite = 1;
+        }
+        e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
+        e = max(e, __shfl_xor_sync(0xffffffffu, e, 2));
+        long long v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = gj_fixed(x[u], e + sg[u]);
+#pragma unroll
+        for (int s = 0; s < NDIG; ++s)
+          *reinterpret_cast<uint2 *>(stage + (size_t)(s * CT * 8 + j) * 8 + 2 * t) =
+              make_uint2(gj_pair(v[0], v[1], s), gj_pair(v[2], v[3], s));
+        if (t == 0) g.rexp[j] = e;
+      }
+      __syncthreads();
+      if (warp < nrb) {
+        for (int ti = 0; ti < nt; ++ti) {
+          float acc[8][4];
+#pragma unroll
+          for (int d = 0; d < 8; ++d)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[d][q] = GJ_MAGIC;
+#pragma unroll
+          for (int u = 0; u < NDIG; ++u) {
+            const uint2 b = *reinterpret_cast<const uint2 *>(
+                stage + (size_t)(u * CT * 8 + ti * 8 + gr) * 8 + 2 * gt);
+#pragma unroll
+            for (int s = 0; s < NDIG; ++s)
+              if (s + u < 8) gj_mma(acc[s + u], a[s], b.x, b.y);
+          }
+          const int tile = c0 + ti;
+          const int c = (tile < k0 / 8 ? tile : tile + 2) * 8 + 2 * gt;
+          const int f0 = g.rexp[ti * 8 + 2 * gt], f1 = g.rexp[ti * 8 + 2 * gt + 1];
+          constexpr int SH = -2 * 1022 - 54;
+          double2 *w0 = reinterpret_cast<double2 *>(A + gj_at(ra, c, ld));
+          double2 *w1 = reinterpret_cast<double2 *>(A + gj_at(rb, c, ld));
+          double2 v0 = *w0, v1 = *w1;
+          v0.x = (pa ? 0.0 : v0.x) + gj_scaled(gj_combine(acc, 0), ea + f0 + SH);
+          v0.y = (pa ? 0.0 : v0.y) + gj_scaled(gj_combine(acc, 1), ea + f1 + SH);
+          v1.x = (pb ? 0.0 : v1.x) + gj_scaled(gj_combine(acc, 2), eb + f0 + SH);
+          v1.y = (pb ? 0.0 : v1.y) + gj_scaled(gj_combine(acc, 3), eb + f1 + SH);
+          *w0 = v0;
+          *w1 = v1;
+        }
+      }
+      __syncthreads();
+    }
+  }
+  // log|det M|, the pivot range and the sign (pivots of rows below N)
+  if (warp < np) {
+    const bool in = tid < N;
+    const double a = in ? fabs(piv) : 1.0;
+    double ls = log(a), mn = in ? a : 1e300, mx = in ? a : 0.0;
+    for (int o = 16; o > 0; o >>= 1) {
+      ls += __shfl_xor_sync(0xffffffffu, ls, o);
+      mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+      mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    const unsigned neg = __ballot_sync(0xffffffffu, in && piv < 0.0);
+    // parity of the row order: pairs of steps taken out of order
+    int inv = 0;
+    if (in)
+      for (int j = tid + 1; j < N; ++j) inv += g.perm[j] < g.perm[tid];
+    const unsigned odd = __ballot_sync(0xffffffffu, inv & 1);
+    if (lane == 0) {
+      g.val[warp] = ls;
+      g.pminw[warp] = mn;
+      g.amax[warp] = mx;
+      g.neg[warp] = __popc(neg) + __popc(odd);
+    }
+  }
+  __syncthreads();
+  if (tid == 0) {
+    double a = 0.0, b = 1e300, c = 0.0;
+    int n = 0;
+    for (int q = 0; q < np; ++q) {
+      a += g.val[q];
+      b = fmin(b, g.pminw[q]);
+      c = fmax(c, g.amax[q]);
+      n += g.neg[q];
+    }
+    g.logdet = g.nonfinite ? nan("") : a;
+    g.pmin = b;
+    g.pmax = c;
+    g.sign = (n & 1) ? -1 : 1;
+  }
+  __syncthreads();
+}
+
+__device__ __forceinline__ double gj_inverse_at(const double *A, int N, int k, int c,
+                                                const GJShared &g) {
+  return A[gj_at(g.perm[k], g.step[c], gj_pad(N))];
+}
+
+// ---------------------------------------------------------------------------
+// The elimination step by step, every multiply-add in FP64.  The blocked form
+// above differs from it in the last bits (about 1e-14 of the inverse, at no
+// larger error).  Two users of the inverse turn last bits into visible
+// differences of a trajectory and keep this form: the mixed form's projected
+// state, whose FP32 inverses have no low words and whose ratios are sums over
+// the operations that cancel, and the mixed form of models with exchange
+// terms, whose SR-CG steps stop before convergence and follow the last bits
+// of the samples (a relative change of 1e-9 in E moves the step by up to 5 %).
+// Threads: 128, or 256 where one CTA fills an SM's shared memory (N > 112).
+// The N^3 multiply-adds keep the FP64 pipe 67 % busy at N = 112, two CTAs per
+// SM; a form with the matrix in registers (16 x 16 threads, one CTA per SM)
+// was slower there, 645 against 465 ms for 608 x 256 inverses: nothing runs
+// under its chain of pivots.
 // In place on an N x N row-major matrix (row stride lda) in shared or global
 // memory.  Two barriers per elimination step:
 //   (P, B) two warps take the pivot of column k from the per-warp
@@ -27,12 +463,13 @@ constexpr int NWARP = NT / 32;
 //       needs no barrier of its own.
 // Entries of the rank-1 update in flight per thread.
 constexpr int GJ_ILP = 4;
+constexpr int ST_WARPS = 8;          // most warps of the step-by-step form
 
-struct GJShared {
-  double val[NWARP];
-  double amax[NWARP];
-  unsigned long long ckey[2][NWARP];   // per-warp pivot candidates (|a| bits) ...
-  int cidx[2][NWARP];                  // ... and their rows, double-buffered by step
+struct GJSteps {
+  double val[ST_WARPS];
+  double amax[ST_WARPS];
+  unsigned long long ckey[2][ST_WARPS];   // per-warp pivot candidates (|a| bits) ...
+  int cidx[2][ST_WARPS];                  // ... and their rows, double-buffered by step
   int bad;
   int sign;
   double logdet;
@@ -42,7 +479,7 @@ struct GJShared {
   double rowk[VMC_MAX_N];   // raw pivot row of the current step
   double coln[VMC_MAX_N];   // column k+1 before the current step's update
   double apiv[VMC_MAX_N];   // |pivot| of every step
-  double pminw[NWARP];
+  double pminw[ST_WARPS];
 };
 
 // |a| as an ordered integer key; NaN below every number (never a pivot)
@@ -52,7 +489,7 @@ __device__ __forceinline__ unsigned long long pivot_key(double a) {
 }
 
 // warp-wide largest key (ties: lowest row); lane 0 records it in slot buf
-__device__ __forceinline__ void pivot_candidates(unsigned long long key, int row, GJShared &g,
+__device__ __forceinline__ void pivot_candidates(unsigned long long key, int row, GJSteps &g,
                                                  int buf) {
   for (int o = 16; o > 0; o >>= 1) {
     const unsigned long long ok = __shfl_xor_sync(0xffffffffu, key, o);
@@ -68,8 +505,10 @@ __device__ __forceinline__ void pivot_candidates(unsigned long long key, int row
   }
 }
 
-__device__ __forceinline__ void gj_invert(double *A, int lda, int N, int *perm, GJShared &g) {
+template <int NTH>   // threads of the CTA
+__device__ __forceinline__ void gj_steps(double *A, int lda, int N, int *perm, GJSteps &g) {
   const int tid = threadIdx.x;
+  constexpr int nth = NTH, nwarp = NTH / 32;
   if (tid == 0) {
     g.logdet = 0.0;
     g.sign = 1;
@@ -81,7 +520,7 @@ __device__ __forceinline__ void gj_invert(double *A, int lda, int N, int *perm, 
   {
     unsigned long long key = 0ull;
     int row = N;
-    for (int i = tid; i < N; i += NT) {
+    for (int i = tid; i < N; i += nth) {
       const unsigned long long kk = pivot_key(A[(size_t)i * lda]);
       if (kk > key) {
         key = kk;
@@ -91,7 +530,7 @@ __device__ __forceinline__ void gj_invert(double *A, int lda, int N, int *perm, 
     pivot_candidates(key, row, g, 0);
   }
   __syncthreads();
-  const int qn = NT / N, rn = NT - (NT / N) * N;
+  const int qn = nth / N, rn = nth - (nth / N) * N;
   auto adv = [&](int &ii, int &cc) {
     ii += qn;
     cc += rn;
@@ -110,7 +549,7 @@ __device__ __forceinline__ void gj_invert(double *A, int lda, int N, int *perm, 
     if (tid < 64) {
       unsigned long long bk = g.ckey[buf][0];
       int p = g.cidx[buf][0];
-      for (int q = 1; q < NWARP; ++q) {
+      for (int q = 1; q < nwarp; ++q) {
         const unsigned long long kq = g.ckey[buf][q];
         const int iq = g.cidx[buf][q];
         if (kq > bk || (kq == bk && iq < p)) {
@@ -166,7 +605,7 @@ __device__ __forceinline__ void gj_invert(double *A, int lda, int N, int *perm, 
     if (k1 < N) {
       unsigned long long key = 0ull;
       int row = N;
-      for (int i = tid; i < N; i += NT) {
+      for (int i = tid; i < N; i += nth) {
         const double v = fma(g.colk[i], g.rowk[k1], g.coln[i]);
         const unsigned long long kk = pivot_key(v);
         const bool t = (i >= k1) & (kk > key);
@@ -216,7 +655,7 @@ __device__ __forceinline__ void gj_invert(double *A, int lda, int N, int *perm, 
   // log|det M| and the pivot range, off the elimination's serial path
   {
     double ls = 0.0, mn = 1e300, mx = 0.0;
-    for (int i = tid; i < N; i += NT) {
+    for (int i = tid; i < N; i += nth) {
       const double a = g.apiv[i];
       ls += log(a);
       mn = fmin(mn, a);
@@ -235,7 +674,7 @@ __device__ __forceinline__ void gj_invert(double *A, int lda, int N, int *perm, 
     __syncthreads();
     if (tid == 0) {
       double a = 0.0, b = 1e300, c = 0.0;
-      for (int q = 0; q < NWARP; ++q) {
+      for (int q = 0; q < nwarp; ++q) {
         a += g.val[q];
         b = fmin(b, g.pminw[q]);
         c = fmax(c, g.amax[q]);
@@ -248,7 +687,7 @@ __device__ __forceinline__ void gj_invert(double *A, int lda, int N, int *perm, 
   for (int k = N - 1; k >= 0; --k) {
     const int p = perm[k];
     if (p == k) continue;   // uniform: perm is shared
-    for (int r = tid; r < N; r += NT) {
+    for (int r = tid; r < N; r += nth) {
       const double t0 = A[(size_t)r * lda + k];
       A[(size_t)r * lda + k] = A[(size_t)r * lda + p];
       A[(size_t)r * lda + p] = t0;
@@ -257,5 +696,8 @@ __device__ __forceinline__ void gj_invert(double *A, int lda, int N, int *perm, 
   }
   __syncthreads();
 }
+
+
+inline int gj_step_threads(int n_max) { return n_max > 112 ? 32 * ST_WARPS : 128; }
 
 }  // namespace vmc_gj

@@ -33,6 +33,7 @@
 #include "vmc_gj.cuh"
 
 #include <math.h>
+#include <type_traits>
 
 namespace {
 
@@ -366,49 +367,68 @@ __device__ void proj_exchange_update(T *Mg, int N, int n, int m, const T *w, con
 // context's precision; log|A_g| and the sign of A_g = sigma_g det M_g kept
 // for the shares (k_proj_shares).  With only_due, walkers whose accepted-move
 // count has not reached due_threshold are skipped.
-template <typename T>
-__global__ void __launch_bounds__(NT) k_proj_build(const SysDev *systems, const int2 *work,
-                                                   int n_work, int Ng, int only_due,
-                                                   int due_threshold) {
+// FP64 inverses by panels above GJ_STEPS_MAX_N, the others and the mixed form's
+// FP32 ones step by step (vmc_gj.cuh has the reasons).
+static bool build_by_panels(int precision, int n_max) {
+  return precision == 0 && n_max > vmc_gj::GJ_STEPS_MAX_N;
+}
+
+// The matrix, with the staged digits of the elimination by panels.
+__host__ __device__ inline size_t build_matrix_bytes(bool panels, int N) {
+  return panels ? vmc_gj::gj_matrix_bytes(N) + vmc_gj::GJ_STAGE_BYTES
+                : pal((size_t)N * ((N % 2) ? N : N + 1) * sizeof(double));
+}
+
+template <typename T, bool PANELS, int NTH>   // NTH as of k_init
+__global__ void __launch_bounds__(NTH, PANELS ? 2 : 0)
+    k_proj_build(const SysDev *systems, const int2 *work, int n_work, int Ng, int only_due,
+                 int due_threshold) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ SysDev S;
-  __shared__ vmc_gj::GJShared gs;
+  using Scratch = typename std::conditional<PANELS, vmc_gj::GJShared, vmc_gj::GJSteps>::type;
+  __shared__ Scratch gs;
   __shared__ int sgm;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, nth = PANELS ? blockDim.x : NTH;
   for (long long item = blockIdx.x; item < (long long)n_work * Ng; item += gridDim.x) {
     __syncthreads();
     const int2 wk = work[item / Ng];
     const int g = (int)(item % Ng);
-    load_sys(&S, systems + wk.x);
     const int w = wk.y;
-    if (only_due && S.acc_since[w] < due_threshold) continue;
+    if (only_due && systems[wk.x].acc_since[w] < due_threshold) continue;
+    load_sys(&S, systems + wk.x);
     const int N = S.N, Ns = S.Ns, Ne = S.Ne;
+    const int P = PANELS ? vmc_gj::gj_pad(N) : N;
     const int ldm = (N % 2) ? N : N + 1;
     double *A = (double *)smem_raw;
-    int *ele = (int *)(A + (size_t)N * ldm);
-    int *perm = ele + Ne;
+    uint32_t *stage = (uint32_t *)(smem_raw + vmc_gj::gj_matrix_bytes(N));
+    int *gsite = (int *)(smem_raw + build_matrix_bytes(PANELS, N));   // Ne, then N for the row order
     const int *inv = S.pinv + (size_t)g * Ns;
     const signed char *sg = S.psgn + (size_t)g * Ns;
-    for (int k = tid; k < Ne; k += NT) ele[k] = S.ele[(size_t)w * Ne + k];
-    if (tid == 0) sgm = 1;
-    __syncthreads();
+    const int *ele = S.ele + (size_t)w * Ne;
+    // the electrons' sites under g^-1, and sigma_g(x), the product of the
+    // operation's signs over the electrons
+    for (int k = tid; k < Ne; k += nth) gsite[k] = inv[ele[k]];
     if (tid < 32) {
-      // sigma_g(x): the product of the operation's signs over the electrons
       int neg = 0;
       for (int k = tid; k < Ne; k += 32) neg += sg[ele[k]] < 0;
       neg = warp_sum(neg);
       if (tid == 0) sgm = (neg & 1) ? -1 : 1;
     }
-    for (int q = tid; q < N * N; q += NT) {
-      const int n = q / N, m = q - n * N;
-      A[n * ldm + m] = S.f64[(size_t)inv[ele[n]] * Ns + inv[ele[N + m]]];
+    __syncthreads();
+    for (int q = tid; q < P * P; q += nth) {
+      const int n = q / P, m = q - n * P;
+      const double f = (n < N && m < N) ? S.f64[(size_t)gsite[n] * Ns + gsite[N + m]]
+                                        : (n == m ? 1.0 : 0.0);
+      A[PANELS ? vmc_gj::gj_at(n, m, P) : n * ldm + m] = f;
     }
     __syncthreads();
-    vmc_gj::gj_invert(A, ldm, N, perm, gs);
+    if constexpr (PANELS) vmc_gj::gj_invert(A, stage, N, gs);
+    else vmc_gj::gj_steps<NTH>(A, ldm, N, gsite + Ne, gs);
     T *dst = proj_minv<T>(S, w, g);
-    for (int q = tid; q < N * N; q += NT) {
+    for (int q = tid; q < N * N; q += nth) {
       const int n = q / N, m = q - n * N;
-      dst[q] = (T)A[n * ldm + m];
+      if constexpr (PANELS) dst[q] = gs.bad ? (T)0 : (T)vmc_gj::gj_inverse_at(A, N, n, m, gs);
+      else dst[q] = gs.bad ? (T)0 : (T)A[n * ldm + m];
     }
     if (tid == 0) {
       const size_t k = (size_t)w * Ng + g;
@@ -955,6 +975,10 @@ size_t vmc_proj_smem(int precision, int N, int Ns, int n_ops) {
                         : proj_layout<float>(N, Ns, n_ops, nullptr, nullptr);
 }
 
+size_t vmc_proj_build_smem(int precision, int N) {
+  return build_matrix_bytes(build_by_panels(precision, N), N) + sizeof(int) * 3 * (size_t)N;
+}
+
 int vmc_proj_occupancy(int precision, size_t smem) {
   int nb = 0;
   if (precision == 0)
@@ -964,20 +988,31 @@ int vmc_proj_occupancy(int precision, size_t smem) {
   return nb;
 }
 
+using BuildKernel = void (*)(const SysDev *, const int2 *, int, int, int, int);
+static BuildKernel build_kernel(int precision, bool panels, int nth) {
+  if (panels) return k_proj_build<double, true, vmc_gj::MAX_THREADS>;
+  if (precision == 0) return k_proj_build<double, false, NT>;
+  return nth == NT ? k_proj_build<float, false, NT>
+                   : k_proj_build<float, false, vmc_gj::MAX_THREADS>;
+}
+
 cudaError_t vmc_proj_set_smem(size_t s_sample, size_t s_build) {
   cudaError_t e;
   if ((e = cudaFuncSetAttribute(k_proj_sample<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_sample))) return e;
   if ((e = cudaFuncSetAttribute(k_proj_sample<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_sample))) return e;
   if ((e = cudaFuncSetAttribute(k_proj_eval<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_sample))) return e;
   if ((e = cudaFuncSetAttribute(k_proj_eval<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_sample))) return e;
-  if ((e = cudaFuncSetAttribute(k_proj_build<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_build))) return e;
-  if ((e = cudaFuncSetAttribute(k_proj_build<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_build))) return e;
+  for (int q = 0; q < 3; ++q)   // FP64 by panels, FP64 and FP32 step by step
+    for (int nth : {NT, vmc_gj::MAX_THREADS})
+      if ((e = cudaFuncSetAttribute(build_kernel(q == 2, q == 0, nth),
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_build)))
+        return e;
   return cudaSuccess;
 }
 
 cudaError_t vmc_launch_proj_build(const SysDev *d_sys, const int2 *d_work, int n_work, int n_ops,
-                                  int precision, int only_due, int due_threshold, size_t smem,
-                                  cudaStream_t st, long long *nl) {
+                                  int precision, int n_max, int only_due, int due_threshold,
+                                  size_t smem, cudaStream_t st, long long *nl) {
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -985,11 +1020,13 @@ cudaError_t vmc_launch_proj_build(const SysDev *d_sys, const int2 *d_work, int n
   const int g1 = (int)(items < 8LL * nsm ? items : 8LL * nsm);
   const int g2 = n_work < 8 * nsm ? n_work : 8 * nsm;
   if (g1 < 1) return cudaSuccess;
+  const bool panels = build_by_panels(precision, n_max);
+  const int nth = panels ? vmc_gj::gj_threads(n_max) : vmc_gj::gj_step_threads(n_max);
+  build_kernel(precision, panels, nth)<<<g1, nth, smem, st>>>(d_sys, d_work, n_work, n_ops, only_due,
+                                                      due_threshold);
   if (precision == 0) {
-    k_proj_build<double><<<g1, NT, smem, st>>>(d_sys, d_work, n_work, n_ops, only_due, due_threshold);
     k_proj_shares<double><<<g2, NT, 0, st>>>(d_sys, d_work, n_work, only_due, due_threshold);
   } else {
-    k_proj_build<float><<<g1, NT, smem, st>>>(d_sys, d_work, n_work, n_ops, only_due, due_threshold);
     k_proj_shares<float><<<g2, NT, 0, st>>>(d_sys, d_work, n_work, only_due, due_threshold);
   }
   *nl += 2;

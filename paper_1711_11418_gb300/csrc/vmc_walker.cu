@@ -31,6 +31,18 @@ __host__ __device__ __forceinline__ size_t minv_bytes(int N, int ldm, int esize)
   return align_up((size_t)N * ldm * esize, 128);
 }
 
+// Shared memory of the from-scratch inverse: the matrix, and the scratch that
+// holds the staged digits of R and, after the elimination, two ints per site.
+// rows: rows of odd stride (step by step, double-float) instead of padded ones.
+__host__ __device__ __forceinline__ size_t init_matrix_bytes(int N, bool rows) {
+  return rows ? align_up((size_t)N * ((N % 2) ? N : N + 1) * sizeof(double), 16)
+              : vmc_gj::gj_matrix_bytes(N);
+}
+__host__ __device__ __forceinline__ size_t init_scratch_bytes(int Ns, bool rows) {
+  const size_t s = align_up(sizeof(int) * (2 * (size_t)Ns + 1), 16);
+  return (rows || s > vmc_gj::GJ_STAGE_BYTES) ? s : vmc_gj::GJ_STAGE_BYTES;
+}
+
 // ---- TMA bulk copies (cp.async.bulk) with an mbarrier, bounded waits ----
 constexpr uint32_t WAIT_LIMIT = 1u << 22;   // try_wait attempts before giving up
 
@@ -2113,31 +2125,33 @@ __global__ void k_expand_mlp(SysDev S) {
   }
 }
 
-// From-scratch inverse of M (Gauss-Jordan with partial pivoting, in place in
-// shared memory: FP64, or double-float by the mixed form's opt-in), log|det M| and its
-// sign, Jastrow field and occupation table.  With only_due, only walkers
-// whose accepted-move count since the last inverse reached due_threshold are
-// rebuilt, and the drift max|M^-1_updated - M^-1_fresh| / max|M^-1_fresh| is
-// recorded.  Work items are taken from the counter *ctr (zeroed by the
-// launcher) one at a time, so the CTAs share the due walkers evenly whatever
-// their positions in the list.
-template <typename T>
-__global__ void __launch_bounds__(NT) k_init(const SysDev *systems, const int2 *work, int n_work,
-                                             int *ctr, int only_due, int due_threshold) {
+// From-scratch inverse of M (Gauss-Jordan with partial pivoting in shared
+// memory: by panels or step by step in FP64, vmc_gj.cuh, or in double-float by
+// the mixed form's opt-in: FORM = VMC_INIT_*), log|det M| and its sign, Jastrow
+// field and occupation table.  With only_due, only walkers whose accepted-move count since the last
+// inverse reached due_threshold are rebuilt, and the drift
+// max|M^-1_updated - M^-1_fresh| / max|M^-1_fresh| is recorded.  Work items
+// are taken from the counter *ctr (zeroed by the launcher) one at a time, so
+// the CTAs share the due walkers evenly whatever their positions in the list.
+// NTH: most threads of the CTA, exactly so many unless by panels.
+template <typename T, int FORM, int NTH>
+__global__ void __launch_bounds__(NTH, FORM == VMC_INIT_BLOCKED ? 2 : 0)
+    k_init(const SysDev *systems, const int2 *work, int n_work, int *ctr, int only_due,
+           int due_threshold) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ SysDev S;
   __shared__ int s_item;
-  __shared__ double red_d[NWARP], red_a[NWARP];
-  // FP64 elimination; the mixed form's opt-in double-float one
-  // (VMC_REBUILD_DOUBLE_FLOAT) shares the scratch
+  constexpr bool DF = FORM == VMC_INIT_DF;
+  constexpr int MW = NTH / 32;
+  __shared__ double red_d[MW], red_a[MW];
   constexpr bool F32 = std::is_same<T, float>::value;
-  __shared__ union {
-    vmc_gj::GJShared d;
-    GJdf f;
-  } gs;
+  using Scratch = typename std::conditional<
+      DF, GJdf, typename std::conditional<FORM == VMC_INIT_BLOCKED, vmc_gj::GJShared, vmc_gj::GJSteps>::type>::type;
+  __shared__ Scratch gs;
+  const int tid = threadIdx.x, nth = FORM == VMC_INIT_BLOCKED ? blockDim.x : NTH;
   auto next_item = [&]() -> int {
     __syncthreads();   // every thread has read the previous item
-    if (threadIdx.x == 0) s_item = atomicAdd(ctr, 1);
+    if (tid == 0) s_item = atomicAdd(ctr, 1);
     __syncthreads();
     return s_item;
   };
@@ -2146,36 +2160,48 @@ __global__ void __launch_bounds__(NT) k_init(const SysDev *systems, const int2 *
     const int w = wk.y;
     if (only_due && systems[wk.x].acc_since[w] < due_threshold) continue;
     load_sys(&S, systems + wk.x);
-    const int N = S.N, Ns = S.Ns, Ne = S.Ne, ldm = S.ldm, tid = threadIdx.x;
-    const bool use_df = F32 && S.rebuild_df;
-    // N x ldm matrix: FP64 words, or (double-float) hi words then lo words
+    const int N = S.N, Ns = S.Ns, Ne = S.Ne, ldm = S.ldm;
+    // the matrix (FP64 words, or hi words then lo words), then scratch: the
+    // staged digits of the elimination, and after it the sites' occupations
     double *A = (double *)smem_raw;
     float *Ah = (float *)smem_raw, *Al = Ah + (size_t)N * ldm;
-    int *ele = (int *)(A + (size_t)N * ldm);        // Ne
-    int *perm = ele + Ne;                            // N
-    for (int k = tid; k < Ne; k += NT) ele[k] = S.ele[(size_t)w * Ne + k];
+    constexpr bool ROWS = FORM != VMC_INIT_BLOCKED;
+    unsigned char *scr = smem_raw + init_matrix_bytes(N, ROWS);
+    int *ele = (int *)(scr + init_scratch_bytes(Ns, ROWS));   // Ne
+    int *perm = ele + Ne;                                     // N (not by panels)
+    for (int k = tid; k < Ne; k += nth) ele[k] = S.ele[(size_t)w * Ne + k];
     __syncthreads();
-    for (int q = tid; q < N * N; q += NT) {
-      const int n = q / N, m = q - n * N;
-      const double f = S.f64[(size_t)ele[n] * Ns + ele[N + m]];
-      if (use_df)
-        df_split(f, Ah[n * ldm + m], Al[n * ldm + m]);
-      else
-        A[n * ldm + m] = f;
+    if constexpr (DF) {
+      for (int q = tid; q < N * N; q += nth) {
+        const int n = q / N, m = q - n * N;
+        df_split(S.f64[(size_t)ele[n] * Ns + ele[N + m]], Ah[n * ldm + m], Al[n * ldm + m]);
+      }
+      __syncthreads();
+      gj_invert_df(Ah, Al, ldm, N, perm, gs);
+    } else if constexpr (FORM == VMC_INIT_STEPS) {
+      for (int q = tid; q < N * N; q += nth) {
+        const int n = q / N, m = q - n * N;
+        A[n * ldm + m] = S.f64[(size_t)ele[n] * Ns + ele[N + m]];
+      }
+      __syncthreads();
+      vmc_gj::gj_steps<NTH>(A, ldm, N, perm, gs);
+    } else {
+      const int P = vmc_gj::gj_pad(N);
+      for (int q = tid; q < P * P; q += nth) {
+        const int n = q / P, m = q - n * P;
+        A[vmc_gj::gj_at(n, m, P)] = (n < N && m < N) ? S.f64[(size_t)ele[n] * Ns + ele[N + m]]
+                                                     : (n == m ? 1.0 : 0.0);
+      }
+      __syncthreads();
+      vmc_gj::gj_invert(A, (uint32_t *)scr, N, gs);
     }
-    __syncthreads();
-    if (use_df)
-      gj_invert_df(Ah, Al, ldm, N, perm, gs.f);
-    else
-      vmc_gj::gj_invert(A, ldm, N, perm, gs.d);
-    const int g_bad = use_df ? gs.f.bad : gs.d.bad;
-    const int g_sign = use_df ? gs.f.sign : gs.d.sign;
-    const double g_logdet = use_df ? gs.f.logdet : gs.d.logdet;
-    const double g_pmin = use_df ? gs.f.pmin : gs.d.pmin;
-    const double g_pmax = use_df ? gs.f.pmax : gs.d.pmax;
-    // the fresh inverse's entry q (FP64 value)
-    auto fresh_at = [&](int q) -> double {
-      return use_df ? (double)Ah[q] + (double)Al[q] : A[q];
+    const int g_bad = gs.bad, g_sign = gs.sign;
+    const double g_logdet = gs.logdet, g_pmin = gs.pmin, g_pmax = gs.pmax;
+    // the fresh inverse's entry (r, c) (FP64 value)
+    auto fresh_at = [&](int r, int c) -> double {
+      if constexpr (DF) return (double)Ah[r * ldm + c] + (double)Al[r * ldm + c];
+      else if constexpr (FORM == VMC_INIT_STEPS) return A[r * ldm + c];
+      else return vmc_gj::gj_inverse_at(A, N, r, c, gs);
     };
     const size_t nb = minv_bytes(N, ldm, sizeof(T));
     T *dst = (T *)((unsigned char *)S.minv + (size_t)w * nb);
@@ -2186,9 +2212,9 @@ __global__ void __launch_bounds__(NT) k_init(const SysDev *systems, const int2 *
     if (!g_bad) {
       if (only_due) {
         double dmax = 0.0, amax = 0.0;
-        for (int q = tid; q < N * N; q += NT) {
+        for (int q = tid; q < N * N; q += nth) {
           const int r = q / N, c = q - r * N;
-          const double fresh = fresh_at(r * ldm + c);
+          const double fresh = fresh_at(r, c);
           const double cur = (double)dst[r * ldm + c] + (dlo ? (double)dlo[r * ldm + c] : 0.0);
           dmax = fmax(dmax, fabs(cur - fresh));
           amax = fmax(amax, fabs(fresh));
@@ -2204,7 +2230,7 @@ __global__ void __launch_bounds__(NT) k_init(const SysDev *systems, const int2 *
         __syncthreads();
         if (tid == 0) {
           double d = 0.0, a = 0.0;
-          for (int q = 0; q < NWARP; ++q) {
+          for (int q = 0; q < nth / 32; ++q) {
             d = fmax(d, red_d[q]);
             a = fmax(a, red_a[q]);
           }
@@ -2213,21 +2239,26 @@ __global__ void __launch_bounds__(NT) k_init(const SysDev *systems, const int2 *
         __syncthreads();
       }
       const bool keep_lo = dlo && S.delay_k <= 1;
-      for (int q = tid; q < N * ldm; q += NT) {
-        if (use_df) {
+      for (int q = tid; q < N * ldm; q += nth) {
+        const int r = q / ldm, c = q - r * ldm;
+        if (c >= N) {   // the padding of a row
+          dst[q] = (T)0;
+          if (dlo) dlo[q] = 0.f;
+        } else if constexpr (DF) {
           dst[q] = Ah[q];
           if (dlo) dlo[q] = keep_lo ? Al[q] : 0.f;
         } else {
-          const T h = (T)A[q];
+          const double a = fresh_at(r, c);
+          const T h = (T)a;
           dst[q] = h;
-          if (dlo) dlo[q] = keep_lo ? (float)(A[q] - (double)h) : 0.f;
+          if (dlo) dlo[q] = keep_lo ? (float)(a - (double)h) : 0.f;
         }
       }
     }
     if (!only_due) {
-      for (int k = tid; k < 2 * Ns; k += NT) S.occ[(size_t)w * 2 * Ns + k] = -1;
+      for (int k = tid; k < 2 * Ns; k += nth) S.occ[(size_t)w * 2 * Ns + k] = -1;
       __syncthreads();
-      for (int k = tid; k < Ne; k += NT) {
+      for (int k = tid; k < Ne; k += nth) {
         const int s = (k >= N) ? 1 : 0;
         S.occ[(size_t)w * 2 * Ns + s * Ns + ele[k]] = k;
       }
@@ -2237,19 +2268,20 @@ __global__ void __launch_bounds__(NT) k_init(const SysDev *systems, const int2 *
       // Jastrow field h_i = sum_{j != i} v_ij (n_j - 1), rebuilt in FP64 on
       // every from-scratch inverse: only sites with n_j != 1 contribute; v is
       // symmetric, so row j is read (coalesced).
-      int *nsite = perm + N;        // [Ns] n_j
+      __syncthreads();              // the staged digits are done with
+      int *nsite = (int *)scr;      // [Ns] n_j
       int *jlist = nsite + Ns;      // [Ns] sites with n_j != 1
       int *jcount = jlist + Ns;     // [1]
       if (tid == 0) *jcount = 0;
-      for (int k = tid; k < Ns; k += NT) nsite[k] = 0;
+      for (int k = tid; k < Ns; k += nth) nsite[k] = 0;
       __syncthreads();
-      for (int k = tid; k < Ne; k += NT) atomicAdd(&nsite[ele[k]], 1);
+      for (int k = tid; k < Ne; k += nth) atomicAdd(&nsite[ele[k]], 1);
       __syncthreads();
-      for (int j = tid; j < Ns; j += NT)
+      for (int j = tid; j < Ns; j += nth)
         if (nsite[j] != 1) jlist[atomicAdd(jcount, 1)] = j;
       __syncthreads();
       const int nl = *jcount;
-      for (int i = tid; i < Ns; i += NT) {
+      for (int i = tid; i < Ns; i += nth) {
         double h = 0.0;
         for (int q = 0; q < nl; ++q) {
           const int j = jlist[q];
@@ -2260,7 +2292,7 @@ __global__ void __launch_bounds__(NT) k_init(const SysDev *systems, const int2 *
       __syncthreads();
     }
     // MLP pre-activations from scratch: h_k = b1_k + sum over electrons of W1[k][c_e]
-    for (int k = tid; k < S.n_hidden; k += NT) {
+    for (int k = tid; k < S.n_hidden; k += nth) {
       const int H = S.n_hidden;
       double h = S.params[S.mlp_base + (size_t)H * 2 * Ns + k];
       for (int e = 0; e < Ne; ++e) h += S.W1T64[(size_t)(ele[e] + (e >= N ? Ns : 0)) * H + k];
@@ -2594,9 +2626,15 @@ size_t vmc_walker_smem(int precision, int N, int Ns, int Np, int H, int kd, int 
                         : walker_layout<float>(N, Ns, al, H, kd, with_lo != 0, nullptr, nullptr);
 }
 
-size_t vmc_init_smem(int N, int Ns) {
-  const int ldm = (N % 2) ? N : N + 1;
-  return (size_t)N * ldm * sizeof(double) + sizeof(int) * (3 * N + 2 * Ns + 1) + 64;
+int vmc_init_form(int precision, int df, int exchange, int n_max) {
+  if (precision != 0 && df) return VMC_INIT_DF;
+  return ((precision != 0 && exchange) || n_max <= vmc_gj::GJ_STEPS_MAX_N) ? VMC_INIT_STEPS
+                                                                           : VMC_INIT_BLOCKED;
+}
+
+size_t vmc_init_smem(int N, int Ns, int form) {
+  const bool rows = form != VMC_INIT_BLOCKED;
+  return init_matrix_bytes(N, rows) + init_scratch_bytes(Ns, rows) + sizeof(int) * 3 * (size_t)N;
 }
 
 // The mixed form's sweep variant for a shared-memory size: the 168-register
@@ -2618,6 +2656,17 @@ int vmc_sample_occupancy(int precision, size_t smem) {
   return nb;
 }
 
+using InitKernel = void (*)(const SysDev *, const int2 *, int, int *, int, int);
+static InitKernel init_kernel(int precision, int form, int nth) {
+  if (precision == 0)
+    return form == VMC_INIT_BLOCKED ? k_init<double, VMC_INIT_BLOCKED, vmc_gj::MAX_THREADS>
+                                    : k_init<double, VMC_INIT_STEPS, NT>;
+  if (form == VMC_INIT_BLOCKED) return k_init<float, VMC_INIT_BLOCKED, vmc_gj::MAX_THREADS>;
+  if (form == VMC_INIT_DF) return k_init<float, VMC_INIT_DF, NT>;
+  return nth == NT ? k_init<float, VMC_INIT_STEPS, NT>
+                   : k_init<float, VMC_INIT_STEPS, vmc_gj::MAX_THREADS>;
+}
+
 cudaError_t vmc_walker_set_smem_limits(size_t s64, size_t s32, size_t sinit) {
   cudaError_t e;
   if ((e = cudaFuncSetAttribute(k_sample<double, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s64))) return e;
@@ -2627,8 +2676,12 @@ cudaError_t vmc_walker_set_smem_limits(size_t s64, size_t s32, size_t sinit) {
   if ((e = cudaFuncSetAttribute(k_eval_ratios<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s32))) return e;
   if ((e = cudaFuncSetAttribute(k_corr<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s64))) return e;
   if ((e = cudaFuncSetAttribute(k_corr<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s32))) return e;
-  if ((e = cudaFuncSetAttribute(k_init<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sinit))) return e;
-  if ((e = cudaFuncSetAttribute(k_init<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sinit))) return e;
+  for (int form : {VMC_INIT_BLOCKED, VMC_INIT_STEPS, VMC_INIT_DF})
+    for (int prec = 0; prec < 2; ++prec)
+      for (int nth : {NT, vmc_gj::MAX_THREADS})
+        if ((e = cudaFuncSetAttribute(init_kernel(prec, form, nth),
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sinit)))
+          return e;
   return cudaSuccess;
 }
 
@@ -2649,26 +2702,24 @@ cudaError_t vmc_launch_expand(const SysDev *h_sys, cudaStream_t st, long long *n
 }
 
 cudaError_t vmc_launch_init(const SysDev *d_sys, const int2 *d_work, int n_work, int *d_ctr,
-                            int precision, int only_due, int due_threshold, size_t smem,
-                            cudaStream_t st, long long *nl) {
+                            int precision, int form, int n_max, int only_due, int due_threshold,
+                            size_t smem, cudaStream_t st, long long *nl) {
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const int nth = form == VMC_INIT_BLOCKED ? vmc_gj::gj_threads(n_max)
+                  : form == VMC_INIT_DF    ? NT
+                                           : vmc_gj::gj_step_threads(n_max);
+  const InitKernel kern = init_kernel(precision, form, nth);
   int per = 1;
-  if (precision == 0)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_init<double>, NT, smem);
-  else
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_init<float>, NT, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, nth, smem);
   if (per < 1) per = 1;
   int grid = nsm * per;
   if (grid > n_work) grid = n_work;
   if (grid < 1) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(d_ctr, 0, sizeof(int), st);
   if (e) return e;
-  if (precision == 0)
-    k_init<double><<<grid, NT, smem, st>>>(d_sys, d_work, n_work, d_ctr, only_due, due_threshold);
-  else
-    k_init<float><<<grid, NT, smem, st>>>(d_sys, d_work, n_work, d_ctr, only_due, due_threshold);
+  kern<<<grid, nth, smem, st>>>(d_sys, d_work, n_work, d_ctr, only_due, due_threshold);
   ++*nl;
   return cudaGetLastError();
 }
