@@ -627,6 +627,20 @@ int create_impl(vmc_ctx **out, int n_sys, const vmc_model *models, const int32_t
       }
       if ((rc = dupload(c, (int **)&d.tgt_j, tj.data(), m.n_hop))) return fail(rc);
       if ((rc = dupload(c, (double **)&d.tgt_t, tt.data(), m.n_hop))) return fail(rc);
+      // and by source site, for the power-Lanczos pairs
+      std::vector<int> sp(Ns + 1, 0), si(m.n_hop);
+      std::vector<double> sv(m.n_hop);
+      for (int k = 0; k < m.n_hop; ++k) sp[m.hop_j[k] + 1]++;
+      for (size_t i = 0; i < Ns; ++i) sp[i + 1] += sp[i];
+      std::vector<int> at(sp.begin(), sp.end() - 1);
+      for (int k = 0; k < m.n_hop; ++k) {
+        const int q = at[m.hop_j[k]]++;
+        si[q] = m.hop_i[k];
+        sv[q] = m.hop_t[k];
+      }
+      if ((rc = dupload(c, (int **)&d.src_ptr, sp.data(), Ns + 1))) return fail(rc);
+      if ((rc = dupload(c, (int **)&d.src_i, si.data(), m.n_hop))) return fail(rc);
+      if ((rc = dupload(c, (double **)&d.src_t, sv.data(), m.n_hop))) return fail(rc);
       if ((rc = dalloc(c, &d.tgt_v64, sizeof(double) * (m.n_hop ? m.n_hop : 1)))) return fail(rc);
       if ((rc = dalloc(c, &d.tgt_v32, sizeof(float) * (m.n_hop ? m.n_hop : 1)))) return fail(rc);
     }
@@ -1449,8 +1463,8 @@ int vmc_lanczos_moments(vmc_ctx *c, int32_t system, double *F1, double *F2, doub
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int prec = c->precision == VMC_FP64 ? 0 : 1;
-  const int grid = std::min(s.W, std::max(1, vmc_lanczos_occupancy(prec, s.Ns)) * nsm);
-  const size_t slot = (vmc_lanczos_slot_bytes(prec, s.Ns, s.N) + 255) / 256 * 256;
+  const int grid = std::min(s.W, std::max(1, vmc_lanczos_occupancy(prec, s.Ns, s.N)) * nsm);
+  const size_t slot = (vmc_lanczos_slot_bytes(prec, s.Ns, s.N, s.dev.n_hop) + 255) / 256 * 256;
   const size_t need = slot * grid + sizeof(double) * (2 * (size_t)s.W + 8);
   if (c->lz_bytes < need) {
     if (c->lz_buf) cudaFree(c->lz_buf);
@@ -1465,7 +1479,7 @@ int vmc_lanczos_moments(vmc_ctx *c, int32_t system, double *F1, double *F2, doub
   double *f1 = (double *)((unsigned char *)c->lz_buf + slot * grid);
   double *f2 = f1 + s.W;
   double *mom = f2 + s.W;
-  CKC(vmc_launch_lanczos(c->d_sys, system, prec, s.Ns, grid, c->lz_buf, f1, f2, s.W, mom, c->st,
+  CKC(vmc_launch_lanczos(c->d_sys, system, prec, s.Ns, s.N, grid, c->lz_buf, f1, f2, s.W, mom, c->st,
                          &c->n_launch));
   if (F1) CKC(cudaMemcpyAsync(F1, f1, sizeof(double) * s.W, cudaMemcpyDeviceToHost, c->st));
   if (F2) CKC(cudaMemcpyAsync(F2, f2, sizeof(double) * s.W, cudaMemcpyDeviceToHost, c->st));

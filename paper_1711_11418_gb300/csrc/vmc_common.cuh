@@ -34,6 +34,9 @@ struct SysDev {
   const int *tgt_term;         // [n_hop] term indices
   const int *tgt_j;            // [n_hop] source site of each grouped term
   const double *tgt_t;         // [n_hop] its t
+  const int *src_ptr;          // [Ns+1] hopping terms grouped by source site j (CSR)
+  const int *src_i;            // [n_hop] target site of each
+  const double *src_t;         // [n_hop] its t
   double *tgt_v64;             // [n_hop] v(j, i) of each grouped term (refreshed with v)
   float *tgt_v32;
   const double *U;
@@ -180,9 +183,9 @@ cudaError_t vmc_launch_proj_eval(const SysDev *d_sys, int sys, int walker, int p
 // First-step power-Lanczos local values and moments (vmc_lanczos.cu): table
 // slot bytes per CTA, and the launch (k_lanczos over the walkers, then the
 // four walker means into moments[4]).
-int vmc_lanczos_occupancy(int precision, int Ns);
-size_t vmc_lanczos_slot_bytes(int precision, int Ns, int N);
-cudaError_t vmc_launch_lanczos(const SysDev *d_sys, int sys, int precision, int Ns, int grid,
+int vmc_lanczos_occupancy(int precision, int Ns, int N);
+size_t vmc_lanczos_slot_bytes(int precision, int Ns, int N, int n_hop);
+cudaError_t vmc_launch_lanczos(const SysDev *d_sys, int sys, int precision, int Ns, int N, int grid,
                                void *slots, double *F1, double *F2, int W, double *moments,
                                cudaStream_t st, long long *n_launch);
 
