@@ -439,6 +439,16 @@ int sr_alloc(vmc_ctx *c, SysHost &s, bool need_S, bool need_ir = false) {
       std::vector<int2> tl(ntile);
       vmc_tc_tile_list(s.Np, tl.data());
       CK(dupload(c, &s.tc_tiles, tl.data(), tl.size()));
+    } else {
+      // the plain form's digits, where there is memory for them (the FP64
+      // kernel builds S otherwise)
+      unsigned char *dg = nullptr;
+      int *em = nullptr;
+      if (dalloc(c, &em, sizeof(int) * s.Np) == VMC_OK &&
+          dalloc(c, &dg, vmc_sr_digits_bytes(rows_cap, s.Np)) == VMC_OK) {
+        s.sr.digits = dg;
+        s.sr.emax = em;
+      }
     }
     s.S_alloc = true;
   }

@@ -37,14 +37,16 @@
 #pragma once
 
 #include "vmc_common.cuh"
+#include "vmc_digits.cuh"
 
 namespace vmc_gj {
 
+using vmc_dig::NDIG;
+using vmc_dig::NOEXP;
+
 constexpr int GB = 16;               // panel width: K of one mma.sync m16n8k16
-constexpr int NDIG = 7;              // 8-bit digits of an operand
 constexpr int CT = 4;                // column tiles (of 8) whose digits are staged at a time
 constexpr int MAX_THREADS = 2 * VMC_MAX_N;
-constexpr int NOEXP = -(1 << 20);    // exponent of a group of zeros
 
 __host__ __device__ inline int gj_pad(int N) { return (N + GB - 1) / GB * GB; }
 // A warp per 16 rows for the update (a thread per row for the panel).
@@ -86,61 +88,11 @@ struct GJShared {
   double logdet, pmin, pmax;   // log|det M|, smallest / largest |pivot|
 };
 
-// ---- 56-bit fixed point in digits -------------------------------------------
-// Biased exponent of x (0: zero or subnormal, taken as zero).
-__device__ __forceinline__ int gj_expo(double x) {
-  return (int)(((unsigned)__double2hiint(x) >> 20) & 0x7ffu);
-}
-
-// x 2^(55 - (e - 1022)) rounded to an integer, |q| <= 2^55, for |x| < 2^(e - 1022),
-// plus 128 in each of the six lower bytes: digit 0 (weight 2^48) is the value of
-// the bits from 48 up, digit s = 1..6 (weight 2^(48 - 8 s)) byte 6 - s less 128.
-__device__ __forceinline__ long long gj_fixed(double x, int e) {
-  const long long b = __double_as_longlong(x);
-  const int ex = (int)((b >> 52) & 0x7ff);
-  const int d = min(max(e - ex, 0), 56);
-  long long m = ((b & 0x000fffffffffffffll) | 0x0010000000000000ll) << 2;   // 55 bits
-  m = (m + ((1ll << d) >> 1)) >> d;
-  if (ex == 0) m = 0;
-  return (b < 0 ? -m : m) + 0x0000808080808080ll;
-}
-
-// Digit s of v as a float (an integer in [-128, 128], exact in BF16): the byte
-// placed under the exponent of 2^23, less 2^23 + 128.
-__device__ __forceinline__ float gj_digit(long long v, int s) {
-  const unsigned hi = (unsigned)(v >> 32), lo = (unsigned)v;
-  if (s == 0) return __int_as_float(0x4B000200 + ((int)hi >> 16)) - 8389120.0f;
-  const unsigned w = s <= 2 ? hi : lo;
-  const unsigned k = s <= 2 ? 2 - s : 6 - s;
-  return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440u + k)) - 8388736.0f;
-}
-// Digits s of two values as a BF16 pair (exact: the upper halves).
-__device__ __forceinline__ uint32_t gj_pair(long long v0, long long v1, int s) {
-  return __byte_perm(__float_as_uint(gj_digit(v0, s)), __float_as_uint(gj_digit(v1, s)), 0x7632u);
-}
-
-// V 2^x as a double (to nearest, ties away from zero; |V| < 2^62).
-__device__ __forceinline__ double gj_scaled(long long V, int x) {
-  const unsigned long long s = (unsigned long long)V & 0x8000000000000000ull;
-  unsigned long long u = (unsigned long long)(V < 0 ? -V : V);
-  const int lz = __clzll((long long)u);
-  const int e = 1023 + 63 - lz + x;
-  // bit 63 set, half of the last of 53 places added (a carry out of the top
-  // reaches the exponent), the leading bit added to the exponent field
-  u = ((u << (lz & 63)) + 0x400ull);
-  const unsigned long long m = (u >> 11) | (u < 0x400ull ? 0x0020000000000000ull : 0ull);
-  unsigned long long b = s | (((unsigned long long)(unsigned)(e - 1) << 52) + m);
-  if (V == 0 || e <= 0) b = 0;
-  if (V != 0 && e >= 2046) b = s | 0x7ff0000000000000ull;
-  return __longlong_as_double((long long)b);
-}
-
 // The accumulators start at 1.5 x 2^23, so that their bits hold the integers.
 constexpr float GJ_MAGIC = 12582912.0f;
 constexpr int GJ_MAGIC_BITS = 0x4B400000;
 
-// Sum of the digit products (bits of the accumulators d = 0..7) in units of
-// 2^(E + F - 54) with T < 2^E, R < 2^F; d = 6 and 7 round into d = 5.
+// The digit products' sum of entry q of a tile (vmc_dig::combine).  |n[d]| < 2^21.
 __device__ __forceinline__ long long gj_combine(const float (&a)[8][4], int q) {
   int n[8];
 #pragma unroll
@@ -150,18 +102,10 @@ __device__ __forceinline__ long long gj_combine(const float (&a)[8][4], int q) {
   return (long long)p0 * 4294967296ll + (long long)p1 * 65536ll + (long long)p2;
 }
 
-__device__ __forceinline__ void gj_mma(float (&c)[4], const uint32_t (&a)[4], uint32_t b0,
-                                       uint32_t b1) {
-  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
 // 1 / x by Newton's iteration from the hardware's 20-bit approximation; very
 // large and small x by the division.
 __device__ __forceinline__ double gj_recip(double x) {
-  const int e = gj_expo(x);
+  const int e = vmc_dig::expo(x);
   if (e < 64 || e > 1982) return 1.0 / x;
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -272,7 +216,7 @@ __device__ __forceinline__ void gj_invert(double *A, uint32_t *stage, int N, GJS
       const int p = g.perm[k0 + l];
       int h = 0;
       for (int c = lane; c < Npad; c += 32)
-        if (c < k0 || c >= k0 + GB) h = max(h, gj_expo(A[gj_at(p, c, ld)]));
+        if (c < k0 || c >= k0 + GB) h = max(h, vmc_dig::expo(A[gj_at(p, c, ld)]));
       h = __reduce_max_sync(0xffffffffu, h);
       if (lane == 0) g.sig[l] = h ? h - 1023 : 0;
     }
@@ -298,7 +242,7 @@ __device__ __forceinline__ void gj_invert(double *A, uint32_t *stage, int N, GJS
       }
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const int e0 = gj_expo(x[0][q]), e1 = gj_expo(x[1][q]);
+        const int e0 = vmc_dig::expo(x[0][q]), e1 = vmc_dig::expo(x[1][q]);
         if (e0) ea = max(ea, e0 + sg[q]);
         if (e1) eb = max(eb, e1 + sg[q]);
         if (e0 == 0x7ff || e1 == 0x7ff) g.nonfinite = 1;
@@ -310,15 +254,15 @@ __device__ __forceinline__ void gj_invert(double *A, uint32_t *stage, int N, GJS
       long long q0[4], q1[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        q0[q] = gj_fixed(x[0][q], ea - sg[q]);
-        q1[q] = gj_fixed(x[1][q], eb - sg[q]);
+        q0[q] = vmc_dig::fixed(x[0][q], ea - sg[q]);
+        q1[q] = vmc_dig::fixed(x[1][q], eb - sg[q]);
       }
 #pragma unroll
       for (int s = 0; s < NDIG; ++s) {
-        a[s][0] = gj_pair(q0[0], q0[1], s);
-        a[s][1] = gj_pair(q1[0], q1[1], s);
-        a[s][2] = gj_pair(q0[2], q0[3], s);
-        a[s][3] = gj_pair(q1[2], q1[3], s);
+        a[s][0] = vmc_dig::pair(q0[0], q0[1], s);
+        a[s][1] = vmc_dig::pair(q1[0], q1[1], s);
+        a[s][2] = vmc_dig::pair(q0[2], q0[3], s);
+        a[s][3] = vmc_dig::pair(q1[2], q1[3], s);
       }
       pa = g.step[ra] >= k0;
       pb = g.step[rb] >= k0;
@@ -339,7 +283,7 @@ __device__ __forceinline__ void gj_invert(double *A, uint32_t *stage, int N, GJS
           const int l = 2 * t + (u & 1) + 8 * (u >> 1);
           x[u] = A[gj_at(g.perm[k0 + l], c, ld)];
           sg[u] = g.sig[l];
-          const int ex = gj_expo(x[u]);
+          const int ex = vmc_dig::expo(x[u]);
           if (ex) e = max(e, ex - sg[u]);
           if (ex == 0x7ff) g.nonfinite = 1;
         }
@@ -347,11 +291,11 @@ __device__ __forceinline__ void gj_invert(double *A, uint32_t *stage, int N, GJS
         e = max(e, __shfl_xor_sync(0xffffffffu, e, 2));
         long long v[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = gj_fixed(x[u], e + sg[u]);
+        for (int u = 0; u < 4; ++u) v[u] = vmc_dig::fixed(x[u], e + sg[u]);
 #pragma unroll
         for (int s = 0; s < NDIG; ++s)
           *reinterpret_cast<uint2 *>(stage + (size_t)(s * CT * 8 + j) * 8 + 2 * t) =
-              make_uint2(gj_pair(v[0], v[1], s), gj_pair(v[2], v[3], s));
+              make_uint2(vmc_dig::pair(v[0], v[1], s), vmc_dig::pair(v[2], v[3], s));
         if (t == 0) g.rexp[j] = e;
       }
       __syncthreads();
@@ -368,19 +312,18 @@ __device__ __forceinline__ void gj_invert(double *A, uint32_t *stage, int N, GJS
                 stage + (size_t)(u * CT * 8 + ti * 8 + gr) * 8 + 2 * gt);
 #pragma unroll
             for (int s = 0; s < NDIG; ++s)
-              if (s + u < 8) gj_mma(acc[s + u], a[s], b.x, b.y);
+              if (s + u < 8) vmc_dig::mma(acc[s + u], a[s], b.x, b.y);
           }
           const int tile = c0 + ti;
           const int c = (tile < k0 / 8 ? tile : tile + 2) * 8 + 2 * gt;
           const int f0 = g.rexp[ti * 8 + 2 * gt], f1 = g.rexp[ti * 8 + 2 * gt + 1];
-          constexpr int SH = -2 * 1022 - 54;
           double2 *w0 = reinterpret_cast<double2 *>(A + gj_at(ra, c, ld));
           double2 *w1 = reinterpret_cast<double2 *>(A + gj_at(rb, c, ld));
           double2 v0 = *w0, v1 = *w1;
-          v0.x = (pa ? 0.0 : v0.x) + gj_scaled(gj_combine(acc, 0), ea + f0 + SH);
-          v0.y = (pa ? 0.0 : v0.y) + gj_scaled(gj_combine(acc, 1), ea + f1 + SH);
-          v1.x = (pb ? 0.0 : v1.x) + gj_scaled(gj_combine(acc, 2), eb + f0 + SH);
-          v1.y = (pb ? 0.0 : v1.y) + gj_scaled(gj_combine(acc, 3), eb + f1 + SH);
+          v0.x = (pa ? 0.0 : v0.x) + vmc_dig::scaled(gj_combine(acc, 0), vmc_dig::unit_expo(ea, f0));
+          v0.y = (pa ? 0.0 : v0.y) + vmc_dig::scaled(gj_combine(acc, 1), vmc_dig::unit_expo(ea, f1));
+          v1.x = (pb ? 0.0 : v1.x) + vmc_dig::scaled(gj_combine(acc, 2), vmc_dig::unit_expo(eb, f0));
+          v1.y = (pb ? 0.0 : v1.y) + vmc_dig::scaled(gj_combine(acc, 3), vmc_dig::unit_expo(eb, f1));
           *w0 = v0;
           *w1 = v1;
         }

@@ -559,6 +559,13 @@ cudaError_t vmc_sr_build_S(const SrWork &w, double shift_rel, double shift_abs, 
                            long long *nl) {
   cudaError_t e = cudaMemsetAsync(w.S, 0, sizeof(double) * (size_t)w.Np * w.Np, st);
   if (e) return e;
+  const size_t n2 = (size_t)w.Np * w.Np;
+  if (w.digits) {
+    if ((e = vmc_sr_syrk_digits(w, w.digits, w.emax, st, nl))) return e;
+    k_mirror_shift<<<(unsigned)((n2 + 255) / 256), 256, 0, st>>>(w.S, w.Np, shift_rel, shift_abs);
+    ++*nl;
+    return cudaGetLastError();
+  }
   const int nt = (w.Np + ST - 1) / ST;
   const int ntiles = nt * (nt + 1) / 2;
   int dev = 0, nsm = 0;
@@ -579,7 +586,6 @@ cudaError_t vmc_sr_build_S(const SrWork &w, double shift_rel, double shift_abs, 
   else
     k_syrk32<<<grid, 256, 0, st>>>((const float *)w.O, w.ldO, w.rows, w.Np, w.obar,
                                    1.0 / w.rows, rps, w.S);
-  const size_t n2 = (size_t)w.Np * w.Np;
   k_mirror_shift<<<(unsigned)((n2 + 255) / 256), 256, 0, st>>>(w.S, w.Np, shift_rel, shift_abs);
   *nl += 2;
   return cudaGetLastError();
