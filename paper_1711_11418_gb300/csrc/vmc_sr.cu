@@ -229,101 +229,165 @@ __global__ void k_mirror_shift(double *S, int Np, double shift_rel, double shift
 }
 
 // Blocked right-looking Cholesky (lower triangle in place), panels of CB
-// columns.  Per panel: k_chol_panel factors the diagonal block and solves the
-// panel below it (L_ij = A_ij L_jj^-T); k_syrk_trailing updates the trailing
-// lower triangle (A -= L L^T) in 32x32 tiles.  FP64 throughput per SM is low
-// on this part, so small tiles keep every SM busy on the late panels.
+// columns.  Per panel: k_chol_panel factors the diagonal block, L_jj L_jj^T,
+// forms L_jj^-1 and with it the panel below (L_ij = A_ij L_jj^-T) and the
+// panel's part of the forward solution L z = g; k_syrk_trailing updates the
+// trailing lower triangle (A -= L L^T) in 32x32 tiles and the rest of the
+// right-hand side.  What bounds it: the chain of n pivots (about 1000 clocks
+// each: a reciprocal, a column, a barrier, eight multiply-adds on a pipe that
+// takes 64 clocks for a warp's) and the FP64 pipe for n^3 / 3 multiply-adds.
+// n = 1069: panels 2.37 -> 0.8 ms, both triangular solves 1.32 -> 0.15 ms.
 constexpr int CB = 32;
+constexpr int PT = 128;    // threads of k_chol_panel
 
-// Cholesky of the nb x nb diagonal block D (lower part, shared memory) by one
-// warp: right-looking, column k scaled by 1/L_kk, then the packed triangle
-// {(r, c): k < c <= r < nb} updated with one entry per lane (the triangle is
-// walked by a linear index, so no lane idles on masked entries).  invd[k]
-// receives 1/L_kk; returns the first non-positive pivot (1-based) or 0.
-__device__ int warp_potrf(double (*D)[CB + 1], double *invd, int nb) {
-  const int lane = threadIdx.x & 31;
-  int bad = 0;
-  for (int k = 0; k < nb; ++k) {
-    if (lane == 0) {
-      double a = D[k][k];
-      if (!(a > 0.0) || !isfinite(a)) {
-        if (!bad) bad = k + 1;
-        a = 1.0;
-      }
-      const double d = sqrt(a);
-      D[k][k] = d;
-      invd[k] = 1.0 / d;
-    }
-    __syncwarp();
-    const double iv = invd[k];
-    if (lane > k && lane < nb) D[lane][k] *= iv;
-    __syncwarp();
-    const int m = nb - k - 1;
-    const int T = m * (m + 1) / 2;
-    for (int q = lane; q < T; q += 32) {
-      int i = (int)((sqrtf(8.0f * (float)q + 1.0f) - 1.0f) * 0.5f);
-      while (i * (i + 1) / 2 > q) --i;
-      while ((i + 1) * (i + 2) / 2 <= q) ++i;
-      const int r = k + 1 + i, c = k + 1 + (q - i * (i + 1) / 2);
-      D[r][c] -= D[r][k] * D[c][k];
-    }
-    __syncwarp();
-  }
-  return __shfl_sync(0xffffffffu, bad, 0);
+// 1 / x by Newton's iteration from the hardware's 20-bit approximation; very
+// large and small x by the division.
+__device__ __forceinline__ double fast_recip(double x) {
+  const int e = (int)(((unsigned)__double2hiint(x) >> 20) & 0x7ffu);
+  if (e < 64 || e > 1982) return 1.0 / x;
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  y = fma(fma(-x, y, 1.0), y, y);
+  return fma(fma(-x, y, 1.0), y, y);
 }
 
-// Panel step: every CTA (one warp) factors the diagonal block in shared
-// memory and solves CB rows of the panel below it, X_i = A_i L_jj^-T, by
-// forward substitution with one row per lane (X_ic = (A_ic - sum_{l<c} X_il
-// L_cl) / L_cc).  CTA 0 records the first non-positive pivot in *info
-// (1-based) and stores the factored block: straight into A when it is the
-// only CTA, else into dblk, from where the trailing update copies it (another
-// CTA may still be reading the block).
-__global__ void __launch_bounds__(32) k_chol_panel(double *A, int n, int j0, int nb, int *info,
-                                                   double *dblk) {
-  __shared__ double D[CB][CB + 1];
-  __shared__ double invd[CB];
-  const int lane = threadIdx.x;
-  for (int r = 0; r < CB; ++r)
-    D[r][lane] = (r < nb && lane <= r) ? A[(size_t)(j0 + r) * n + j0 + lane] : (r == lane ? 1.0 : 0.0);
-  __syncwarp();
-  const int bad = warp_potrf(D, invd, nb);
-  if (blockIdx.x == 0) {
-    const bool direct = gridDim.x == 1;
-    for (int r = 0; r < nb; ++r) {
-      if (lane > r) continue;
-      if (direct) A[(size_t)(j0 + r) * n + j0 + lane] = D[r][lane];
-      else dblk[r * nb + lane] = D[r][lane];
-    }
-    if (lane == 0 && bad && *info == 0) *info = j0 + bad;
+// Panel step.  Every CTA factors the nb x nb diagonal block redundantly, lane =
+// row, warp w the columns w, w + 4, ...: elimination without square roots
+// (A = L1 D L1^T, L1 unit) applied to the identity beside it, which gives
+// W1 = L1^-1; L_jj = L1 D^1/2 and W = D^-1/2 W1 = L_jj^-1.  Then four threads
+// to a row form X_i = A_i W^T for CB rows below.  CTA 0 records the first
+// non-positive pivot in *info (1-based), stores W, the panel of the forward
+// solution z = W y, and the factored block: straight into A when it is the only
+// CTA, else into dblk, from where the trailing update copies it (another CTA
+// may still be reading the block).
+__global__ void __launch_bounds__(PT) k_chol_panel(double *A, int n, int j0, int nb, int *info,
+                                                   double *dblk, double *Wout, const double *y,
+                                                   double *z) {
+  __shared__ double Ls[CB][CB + 1], Ws[CB][CB + 1];
+  __shared__ double mcol[2][CB], acol[2][CB];   // multipliers, column before scaling
+  __shared__ double dg[CB], sq[CB], rs[CB];
+  __shared__ int bad_sh;
+  const int tid = threadIdx.x, r = tid & 31, w = tid >> 5;
+  if (tid == 0) bad_sh = 0;
+  double a[CB / 4], v[CB / 4];
+#pragma unroll
+  for (int j = 0; j < CB / 4; ++j) {
+    const int c = w + 4 * j;
+    a[j] = (r < nb && c <= r) ? A[(size_t)(j0 + r) * n + j0 + c] : (r == c ? 1.0 : 0.0);
+    v[j] = (r == c) ? 1.0 : 0.0;
   }
-  const int i = j0 + nb + blockIdx.x * CB + lane;
-  if (i >= n) return;
-  double *row = A + (size_t)i * n + j0;
+  // this thread's row of the panel below, fetched while the block is factored
+  const int i = j0 + nb + blockIdx.x * CB + (tid >> 2);
+  const bool row_ok = blockIdx.x * CB + (tid >> 2) < n - j0 - nb;
   double x[CB];
 #pragma unroll
-  for (int c = 0; c < CB; ++c) x[c] = (c < nb) ? row[c] : 0.0;
+  for (int l = 0; l < CB; ++l) x[l] = (row_ok && l < nb) ? A[(size_t)i * n + j0 + l] : 0.0;
+  __syncthreads();
 #pragma unroll
-  for (int c = 0; c < CB; ++c) {
-    if (c < nb) {
-      double v = x[c];
+  for (int k = 0; k < CB; ++k) {
+    const int b = k & 1;
+    if (w == (k & 3)) {
+      double piv = __shfl_sync(0xffffffffu, a[k >> 2], k);
+      if (!(piv > 0.0) || !isfinite(piv)) {
+        if (r == 0 && !bad_sh) bad_sh = k + 1;
+        piv = 1.0;
+      }
+      const double ip = fast_recip(piv);
+      const double m = r > k ? a[k >> 2] * ip : 0.0;
+      acol[b][r] = a[k >> 2];
+      mcol[b][r] = m;
+      a[k >> 2] = r == k ? 1.0 : m;   // column k of L1
+      if (r == 0) dg[k] = piv;
+    }
+    __syncthreads();
+    const double m = mcol[b][r];
 #pragma unroll
-      for (int l = 0; l < c; ++l) v -= x[l] * D[c][l];
-      x[c] = v * invd[c];
+    for (int j = k >> 2; j < CB / 4; ++j) {
+      const int c = w + 4 * j;
+      if (c > k) a[j] = fma(-m, acol[b][c], a[j]);   // rows r >= c matter
+    }
+#pragma unroll
+    for (int j = 0; j <= (k >> 2); ++j) {
+      const double vk = __shfl_sync(0xffffffffu, v[j], k);
+      if (w + 4 * j <= k) v[j] = fma(-m, vk, v[j]);
     }
   }
+  if (w == 0) {
+    const double d = dg[r];
+    const double s = sqrt(d);
+    sq[r] = s;
+    rs[r] = 1.0 / s;
+  }
+  __syncthreads();
 #pragma unroll
-  for (int c = 0; c < CB; ++c)
-    if (c < nb) row[c] = x[c];
+  for (int j = 0; j < CB / 4; ++j) {
+    const int c = w + 4 * j;
+    Ls[r][c] = c <= r ? a[j] * sq[c] : 0.0;
+    Ws[r][c] = c <= r ? v[j] * rs[r] : 0.0;
+  }
+  __syncthreads();
+  if (blockIdx.x == 0) {
+    const bool direct = gridDim.x == 1;
+    for (int q = tid; q < CB * CB; q += PT) {
+      const int rr = q / CB, c = q % CB;
+      Wout[q] = Ws[rr][c];
+      if (rr < nb && c <= rr) {
+        if (direct) A[(size_t)(j0 + rr) * n + j0 + c] = Ls[rr][c];
+        else dblk[rr * nb + c] = Ls[rr][c];
+      }
+    }
+    if (tid == 0 && bad_sh && *info == 0) *info = j0 + bad_sh;
+    if (w == 3) {
+      double s0 = 0.0, s1 = 0.0;
+      for (int l = 0; l < nb; l += 2) {
+        s0 = fma(Ws[r][l], y[j0 + l], s0);
+        if (l + 1 < nb) s1 = fma(Ws[r][l + 1], y[j0 + l + 1], s1);
+      }
+      if (r < nb) z[j0 + r] = s0 + s1;
+    }
+  }
+  if (!row_ok) return;
+  const int q = tid & 3;
+#pragma unroll
+  for (int j = 0; j < CB / 4; ++j) {
+    const int c = q + 4 * j;
+    double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+    for (int l = 0; l < 4 * j + 4; l += 2) {   // W is lower triangular: l <= c
+      s0 = fma(x[l], Ws[c][l], s0);
+      s1 = fma(x[l + 1], Ws[c][l + 1], s1);
+    }
+    if (c < nb) A[(size_t)i * n + j0 + c] = s0 + s1;
+  }
 }
 
 // Trailing update A[i][k] -= sum_l L[i][j0+l] L[k][j0+l] for j1 <= k <= i < n
 // (j1 = j0 + nb): one 32x32 lower tile per CTA, tile (bi, bj) with bj <= bi
 // decoded from the linear block index.  With copy_diag, CTA 0 also stores
 // the factored diagonal block from dblk (no CTA here reads that block).
+// CTAs from n_tiles on take the panel out of the right-hand side instead:
+// y_k -= sum_l L_{k,j0+l} z_{j0+l}, 256 rows k each.
 __global__ void __launch_bounds__(256) k_syrk_trailing(double *A, int n, int j0, int nb,
-                                                       int copy_diag, const double *dblk) {
+                                                       int copy_diag, const double *dblk,
+                                                       int n_tiles, double *y, const double *z) {
   const int j1 = j0 + nb;
+  if (blockIdx.x >= n_tiles) {
+    __shared__ double zp[CB];
+    if (threadIdx.x < CB) zp[threadIdx.x] = threadIdx.x < nb ? z[j0 + threadIdx.x] : 0.0;
+    __syncthreads();
+    const int k = j1 + (blockIdx.x - n_tiles) * 256 + threadIdx.x;
+    if (k < n) {
+      const double *row = A + (size_t)k * n + j0;
+      double s0 = 0.0, s1 = 0.0;
+#pragma unroll 8
+      for (int l = 0; l < CB; l += 2) {
+        if (l < nb) s0 = fma(row[l], zp[l], s0);
+        if (l + 1 < nb) s1 = fma(row[l + 1], zp[l + 1], s1);
+      }
+      y[k] -= s0 + s1;
+    }
+    return;
+  }
   if (copy_diag && blockIdx.x == 0)
     for (int q = threadIdx.x; q < nb * nb; q += 256) {
       const int r = q / nb, c = q % nb;
@@ -362,79 +426,45 @@ __global__ void __launch_bounds__(256) k_syrk_trailing(double *A, int n, int j0,
     }
 }
 
-// Triangular solves L y = b and L^T x = y, one launch per panel of CB
-// unknowns and direction.  Every CTA stages the panel's diagonal block and
-// solves it redundantly with one unknown per lane (column sweep: lane k
-// finishes its unknown and broadcasts it, the others subtract), then applies
-// the panel to its share of the remaining entries.  The right-hand side is
-// read from one vector and the finished panel written to another, so no CTA
-// reads a value another CTA of the same launch writes.
-//   forward:  rows i >= p0 + nb: y_i -= sum_l L_{i,p0+l} z_{p0+l}   (warp per row);
-//             CTA 0 writes z[p0 .. p0+nb).
-//   backward: rows i < p0:       y_i -= sum_l L_{p0+l,i} x_{p0+l}   (thread per row);
-//             CTA 0 writes x[p0 .. p0+nb).
-constexpr int SV_ROWS = 64;    // forward rows per CTA (8 warps x 8 rows)
-constexpr int SV_COLS = 256;   // backward rows per CTA (one per thread)
+// Backward solve L^T x = z, one launch per panel of CB unknowns, last first:
+// every CTA forms x_p = W^T z_p (W = L_pp^-1 of the factorisation; eight warps
+// share the sums), then takes the panel out of its share of the entries above,
+// z_i -= sum_l L_{p0+l,i} x_{p0+l} for i < p0 (thread per entry).  z is read
+// and x written to another vector, so no CTA reads what another one writes.
+constexpr int SV_COLS = 256;
 
-__device__ __forceinline__ double panel_solve_lane(const double (*Dg)[CB + 1], double v, int nb,
-                                                   bool transpose) {
-  const int lane = threadIdx.x & 31;
-  if (!transpose) {
-    for (int k = 0; k < nb; ++k) {
-      if (lane == k) v /= Dg[k][k];
-      const double xk = __shfl_sync(0xffffffffu, v, k);
-      if (lane > k) v -= Dg[lane][k] * xk;
-    }
-  } else {
-    for (int k = nb - 1; k >= 0; --k) {
-      if (lane == k) v /= Dg[k][k];
-      const double xk = __shfl_sync(0xffffffffu, v, k);
-      if (lane < k) v -= Dg[k][lane] * xk;
-    }
-  }
-  return v;
-}
-
-__global__ void __launch_bounds__(256) k_trsv_panel(const double *L, int n, int p0, int fwd,
-                                                    double *y, double *out) {
-  __shared__ double Dg[CB][CB + 1];
-  __shared__ double xp[CB];
+__global__ void __launch_bounds__(SV_COLS) k_trsv_back(const double *L, int n, int p0,
+                                                       const double *W, double *z, double *x) {
+  __shared__ double part[8][CB], xp[CB];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nb = min(CB, n - p0);
-  for (int q = tid; q < CB * CB; q += 256) {
-    const int r = q / CB, c = q % CB;
-    Dg[r][c] = (r < nb && c <= r) ? L[(size_t)(p0 + r) * n + p0 + c] : (r == c ? 1.0 : 0.0);
+  double s = 0.0;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int rr = warp * 4 + u;
+    if (rr < nb) s = fma(W[rr * CB + lane], z[p0 + rr], s);   // W[rr][lane] = 0 for rr < lane
   }
+  part[warp][lane] = s;
   __syncthreads();
   if (warp == 0) {
-    double v = lane < nb ? y[p0 + lane] : 0.0;
-    v = panel_solve_lane(Dg, v, nb, !fwd);
-    xp[lane] = lane < nb ? v : 0.0;
-    if (blockIdx.x == 0 && lane < nb) out[p0 + lane] = v;
+    double t = part[0][lane];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) t += part[k][lane];
+    xp[lane] = lane < nb ? t : 0.0;
+    if (blockIdx.x == 0 && lane < nb) x[p0 + lane] = t;
   }
   __syncthreads();
-  if (fwd) {
-    const int r0 = p0 + nb + blockIdx.x * SV_ROWS;
-    for (int i = r0 + warp; i < min(n, r0 + SV_ROWS); i += 8) {
-      double s = (lane < nb) ? L[(size_t)i * n + p0 + lane] * xp[lane] : 0.0;
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) y[i] -= s;
+  const int i = blockIdx.x * SV_COLS + tid;
+  if (i < p0) {
+    double s0 = 0.0, s1 = 0.0;
+#pragma unroll 8
+    for (int l = 0; l < CB; l += 2) {
+      if (l < nb) s0 = fma(L[(size_t)(p0 + l) * n + i], xp[l], s0);
+      if (l + 1 < nb) s1 = fma(L[(size_t)(p0 + l + 1) * n + i], xp[l + 1], s1);
     }
-  } else {
-    const int i = blockIdx.x * SV_COLS + tid;
-    if (i < p0) {
-      double s0 = 0.0, s1 = 0.0;
-      int l = 0;
-      for (; l + 2 <= nb; l += 2) {
-        s0 += L[(size_t)(p0 + l) * n + i] * xp[l];
-        s1 += L[(size_t)(p0 + l + 1) * n + i] * xp[l + 1];
-      }
-      if (l < nb) s0 += L[(size_t)(p0 + l) * n + i] * xp[l];
-      y[i] -= s0 + s1;
-    }
+    z[i] -= s0 + s1;
   }
 }
-
 
 // t = O v (one warp per row)
 template <typename TO>
@@ -591,38 +621,36 @@ cudaError_t vmc_sr_build_S(const SrWork &w, double shift_rel, double shift_abs, 
   return cudaGetLastError();
 }
 
-// The launch sequence of the factorisation and both solves: 2 launches per
-// panel plus the solve.  Pointers are fixed for the life of the work area, so
-// the sequence is captured once into a CUDA graph and replayed.
+// The launch sequence of the factorisation (with the forward solve) and the
+// backward solve: three launches per panel.  Pointers are fixed for the life of
+// the work area, so the sequence is captured once into a CUDA graph and
+// replayed.
 static void chol_sequence(const SrWork &w, cudaStream_t st) {
   const int n = w.Np;
   cudaMemsetAsync(w.info, 0, sizeof(int), st);
+  // right-hand side y (= w.p, starts as g) -> z (= w.w), panel by panel
+  cudaMemcpyAsync(w.p, w.g, sizeof(double) * n, cudaMemcpyDeviceToDevice, st);
   for (int j0 = 0; j0 < n; j0 += CB) {
     const int nb = n - j0 < CB ? n - j0 : CB;
     const int rem = n - j0 - nb;
     const int pg = rem > 0 ? (rem + CB - 1) / CB : 1;
-    k_chol_panel<<<pg, 32, 0, st>>>(w.S, n, j0, nb, w.info, w.dblk);
+    double *W = w.dinv + (size_t)(j0 / CB) * CB * CB;
+    k_chol_panel<<<pg, PT, 0, st>>>(w.S, n, j0, nb, w.info, w.dblk, W, w.p, w.w);
     if (rem > 0) {
-      const int nt = (rem + 31) / 32;
-      k_syrk_trailing<<<nt * (nt + 1) / 2, 256, 0, st>>>(w.S, n, j0, nb, pg > 1, w.dblk);
+      const int nt = (rem + 31) / 32, tiles = nt * (nt + 1) / 2;
+      k_syrk_trailing<<<tiles + (rem + 255) / 256, 256, 0, st>>>(w.S, n, j0, nb, pg > 1, w.dblk,
+                                                                 tiles, w.p, w.w);
     }
-  }
-  // forward: y (= w.p, starts as g) -> z (= w.w); backward: z -> x.
-  cudaMemcpyAsync(w.p, w.g, sizeof(double) * n, cudaMemcpyDeviceToDevice, st);
-  for (int p0 = 0; p0 < n; p0 += CB) {
-    const int rem = n - p0 - (n - p0 < CB ? n - p0 : CB);
-    const int grid = rem > 0 ? (rem + SV_ROWS - 1) / SV_ROWS : 1;
-    k_trsv_panel<<<grid, 256, 0, st>>>(w.S, n, p0, 1, w.p, w.w);
   }
   for (int p0 = ((n - 1) / CB) * CB; p0 >= 0; p0 -= CB) {
     const int grid = p0 > 0 ? (p0 + SV_COLS - 1) / SV_COLS : 1;
-    k_trsv_panel<<<grid, 256, 0, st>>>(w.S, n, p0, 0, w.w, w.x);
+    k_trsv_back<<<grid, SV_COLS, 0, st>>>(w.S, n, p0, w.dinv + (size_t)(p0 / CB) * CB * CB, w.w, w.x);
   }
 }
 
 static long long chol_launches(int n) {
   long long c = 0;
-  for (int j0 = 0; j0 < n; j0 += CB) c += (n - j0 > CB) ? 4 : 3;
+  for (int j0 = 0; j0 < n; j0 += CB) c += (n - j0 > CB) ? 3 : 2;
   return c;
 }
 

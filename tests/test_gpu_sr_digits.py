@@ -1,6 +1,7 @@
 """The plain form's overlap matrix from 8-bit digit products, at the edges of
 its tiles (64 parameters, 128 samples) and slabs, with columns of zeros, of one
-value, and with entries far above the rest."""
+value, and with entries far above the rest; and the Cholesky solve at the edges
+of its 32-column panels."""
 import numpy as np
 import pytest
 
@@ -64,3 +65,37 @@ def test_overlap_matrix_in_slabs():
     X = O[:, idx] - O[:, idx].mean(0)
     ref = X.T @ X / rows
     assert np.abs(S[np.ix_(idx, idx)] - ref).max() <= 1e-13 * np.abs(np.diag(ref)).max()
+
+
+@pytest.mark.parametrize("Np", [17, 31, 32, 33, 63, 64, 65, 96, 97, 300])
+def test_cholesky_at_panel_edges(Np):
+    rows = 3 * Np + 40
+    p = problem(Np - 1)
+    rng = np.random.default_rng(Np)
+    O = rng.standard_normal((rows, Np)) * np.exp(rng.standard_normal((1, Np)))
+    E = rng.standard_normal(rows) + O[:, :5].sum(1)
+    with vmc.Context(p, -(-rows // 4), seed=1, precision=vmc.FP64, max_samples=4) as ctx:
+        ctx.set_samples(E, O)
+        S, g = ctx.get_sr_matrices(1e-3, 1e-4)
+        p0 = ctx.get_params()
+        ctx.sr_step(1.0, 1e-3, 1e-4, solver=vmc.CHOLESKY)
+        x = p0 - ctx.get_params()
+    ref = np.linalg.solve(S, g)
+    # |dx| <= const n eps cond |x| for Cholesky; the step is read off parameters of order 1
+    cond = np.linalg.cond(S)
+    assert np.linalg.norm(x - ref) <= 16 * Np * 2.3e-16 * cond * np.linalg.norm(ref) + 1e-15 * np.sqrt(Np) * 4
+
+
+def test_cholesky_reports_a_matrix_that_is_not_positive_definite():
+    Np, rows = 70, 20          # rank deficient, no shift: a pivot is 0 up to rounding
+    p = problem(Np - 1)
+    rng = np.random.default_rng(1)
+    O = np.zeros((rows, Np))
+    O[:, :40] = rng.standard_normal((rows, 40))   # 30 columns of zeros: pivots exactly 0
+    with vmc.Context(p, rows, seed=1, precision=vmc.FP64) as ctx:
+        ctx.set_samples(rng.standard_normal(rows), O)
+        p0 = ctx.get_params()
+        with pytest.raises(vmc.VmcError) as e:
+            ctx.sr_step(0.1, 0.0, 0.0, solver=vmc.CHOLESKY)
+        assert e.value.code == -4
+        assert np.array_equal(ctx.get_params(), p0)
