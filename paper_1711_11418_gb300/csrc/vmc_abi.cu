@@ -462,8 +462,8 @@ int sr_alloc(vmc_ctx *c, SysHost &s, bool need_S, bool need_ir = false) {
   if (need_ir && !s.sr.S32) {
     SrWork &w = s.sr;
     CK(dalloc(c, &w.S32, sizeof(float) * (size_t)s.Np * s.Np));
-    CK(dalloc(c, &w.gjP, sizeof(float) * 32 * 32));
-    CK(dalloc(c, &w.gjC, sizeof(float) * (size_t)(s.Np + 64) * 32));
+    CK(dalloc(c, &w.gjR, sizeof(float) * 64 * (size_t)s.Np));
+    CK(dalloc(c, &w.gjC, sizeof(float) * 64 * (size_t)s.Np));
     CK(dalloc(c, &w.rs32, sizeof(float) * s.Np));
     CK(dalloc(c, &w.dsc, sizeof(double) * s.Np));
     CK(dalloc(c, &w.irflag, sizeof(int) * 4));

@@ -211,7 +211,7 @@ struct SrWork {
   void *chol_graph;            // cudaGraphExec_t of the Cholesky factor + solve (lazily built)
   // mixed-precision iterative refinement (vmc_sr_mixed.cu)
   float *S32;                  // [Np*Np] scaled S~, inverted in place
-  float *gjP, *gjC;            // [32*32] pivot-block inverse, [Np*32] column block
+  float *gjR, *gjC;            // [2][32*Np] rows and columns of a pivot block and the next
   float *rs32;                 // [Np] scaled residual
   double *dsc;                 // [Np] S~_kk^-1/2
   int *irflag;                 // [4] converged, unusable, steps

@@ -95,14 +95,31 @@ __global__ void k_sum_parts(const double *part, int nparts, int Np, double scale
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= Np || (done && *done)) return;
   double s = 0.0;
-  for (int c = 0; c < nparts; ++c) s += part[(size_t)c * Np + k];
+  int c = 0;
+  for (; c + 8 <= nparts; c += 8) {   // one chain of adds, eight loads ahead of it
+    double x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) x[u] = part[(size_t)(c + u) * Np + k];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s += x[u];
+  }
+  for (; c < nparts; ++c) s += part[(size_t)c * Np + k];
   out[k] = s * scale;
 }
 
 __global__ void k_mean_vec(const double *v, int n, double *out) {
   __shared__ double red[256];
   double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s += v[i];
+  // one chain of adds per thread in order, sixteen loads ahead of it
+  int i = threadIdx.x;
+  for (; i + 15 * 256 < n; i += 16 * 256) {
+    double x[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) x[u] = v[i + 256 * u];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) s += x[u];
+  }
+  for (; i < n; i += 256) s += v[i];
   red[threadIdx.x] = s;
   __syncthreads();
   for (int o = blockDim.x / 2; o > 0; o >>= 1) {

@@ -30,126 +30,148 @@ __global__ void k_ir_diag(const double *S, int n, double *dsc, int *flag) {
   }
 }
 
-__global__ void k_ir_scale(const double *S, int n, const double *dsc, float *A) {
+// The scaled matrix, and its first GB rows and columns beside it (k_gj_step)
+__global__ void k_ir_scale(const double *S, int n, const double *dsc, float *A, float *R, float *C) {
   const size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= (size_t)n * n) return;
   const int i = (int)(q / n), j = (int)(q % n);
-  A[q] = (float)(dsc[i] * S[q] * dsc[j]);
+  const float a = (float)(dsc[i] * S[q] * dsc[j]);
+  A[q] = a;
+  if (i < GB) R[(size_t)i * n + j] = a;
+  if (j < GB) C[(size_t)i * GB + j] = a;
 }
 
-// In-place inverse of the nb x nb block D (padded with the identity to GB)
-// by Gauss-Jordan elimination without pivoting (the scaled matrix is
-// symmetric positive definite), 256 threads.
-__device__ void block_invert(float (*D)[GB + 1], float *rowk, float *colk) {
-  const int tid = threadIdx.x;
+// In-place inverse of the GB x GB block D by Gauss-Jordan elimination without
+// pivoting (the scaled matrix is symmetric positive definite), 256 threads:
+// thread = row tid / 8, columns tid % 8 + 8 j, in registers; one barrier per
+// step, at which the next pivot row and column are published.
+__device__ __forceinline__ void block_invert(float (*D)[GB + 1], float (*rowk)[GB],
+                                             float (*colk)[GB]) {
+  const int tid = threadIdx.x, r = tid >> 3, q = tid & 7;
+  float d[GB / 8];
+#pragma unroll
+  for (int j = 0; j < GB / 8; ++j) d[j] = D[r][q + 8 * j];
+  if (r == 0)
+#pragma unroll
+    for (int j = 0; j < GB / 8; ++j) rowk[0][q + 8 * j] = d[j];
+  if (q == 0) colk[0][r] = d[0];
+  __syncthreads();
+#pragma unroll
   for (int k = 0; k < GB; ++k) {
-    if (tid < GB) {
-      rowk[tid] = D[k][tid];
-      colk[tid] = D[tid][k];
+    const float *rk = rowk[k & 1], *ck = colk[k & 1];
+    const float ip = 1.0f / rk[k];
+    const float m = ck[r] * ip;
+#pragma unroll
+    for (int j = 0; j < GB / 8; ++j) {
+      const int c = q + 8 * j;
+      const float row = rk[c];
+      if (r == k) d[j] = c == k ? ip : row * ip;
+      else d[j] = c == k ? -m : d[j] - m * row;
     }
-    __syncthreads();
-    const float ip = 1.0f / rowk[k];
-    for (int q = tid; q < GB * GB; q += 256) {
-      const int r = q / GB, c = q % GB;
-      if (r == k && c == k) D[r][c] = ip;
-      else if (r == k) D[r][c] = rowk[c] * ip;
-      else if (c == k) D[r][c] = -colk[r] * ip;
-      else D[r][c] -= colk[r] * rowk[c] * ip;
+    if (k + 1 < GB) {
+      if (r == k + 1)
+#pragma unroll
+        for (int j = 0; j < GB / 8; ++j) rowk[(k + 1) & 1][q + 8 * j] = d[j];
+      if (q == ((k + 1) & 7)) colk[(k + 1) & 1][r] = d[(k + 1) >> 3];
     }
     __syncthreads();
   }
+#pragma unroll
+  for (int j = 0; j < GB / 8; ++j) D[r][q + 8 * j] = d[j];
+  __syncthreads();
 }
 
-// Gauss-Jordan step on pivot block K = [k0, k0 + nb): every CTA inverts A_KK
-// into shared memory (CTA 0 stores it in P); CTA b then forms the new row
-// block A_Kj <- P A_Kj for its columns j in [GT b, GT b + GT) \ K and copies
-// the old column block C_i = A_iK for its rows i in the same range.
-__global__ void __launch_bounds__(256) k_gj_row(float *A, int n, int k0, int nb, float *P, float *C) {
+// Gauss-Jordan step on pivot block K = [k0, k0 + nb), one GT x GT tile of A per
+// CTA, in place.  R (GB x n) and C (n x GB) hold the rows and columns of K as
+// they were before the step, Rn and Cn receive those of the next block, so a
+// step reads nothing of A but its own tile and needs one launch.  Every CTA
+// inverts A_KK (P) and forms its columns of the new row block, B = P A_Kj, or P
+// itself for the columns of K; then
+//   i in K:      A_ij <- B
+//   i not in K:  A_ij <- (j in K ? 0 : A_ij) - sum_l C_il B_lj.
+// What bounds it: latency (a 32-step inversion, two small products, one tile);
+// n = 1069: 39 us in two launches per step -> 9.5 us.
+__global__ void __launch_bounds__(256) k_gj_step(float *A, int n, int k0, int nb, const float *R,
+                                                 const float *C, float *Rn, float *Cn) {
   __shared__ float D[GB][GB + 1];
-  __shared__ float R[GB][GT + 1];
-  __shared__ float rowk[GB], colk[GB];
-  const int tid = threadIdx.x;
-  for (int q = tid; q < GB * GB; q += 256) {
-    const int r = q / GB, c = q % GB;
-    D[r][c] = (r < nb && c < nb) ? A[(size_t)(k0 + r) * n + k0 + c] : (r == c ? 1.0f : 0.0f);
+  __shared__ float Bs[GB][GT + 1];
+  __shared__ float Cs[GT][GB + 1];
+  __shared__ float rowk[2][GB], colk[2][GB];
+  const int nt = (n + GT - 1) / GT;
+  const int i0 = (blockIdx.x / nt) * GT, j0 = (blockIdx.x % nt) * GT, tid = threadIdx.x;
+  const int tx = tid & 15, ty = tid >> 4;
+  auto inK = [&](int x) { return x >= k0 && x < k0 + nb; };
+  // the tile and the operands are fetched while A_KK is inverted
+  float a[4][4], rv[8];
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const int i = i0 + ty + 16 * u, j = j0 + tx + 16 * v;
+      a[u][v] = (i < n && j < n && !inK(j)) ? A[(size_t)i * n + j] : 0.0f;
+    }
+  const int bl = tid >> 3, bc = tid & 7;   // B: row bl, columns bc + 8 u
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int j = j0 + bc + 8 * u;
+    rv[u] = (bl < nb && j < n) ? R[(size_t)bl * n + j] : 0.0f;
+  }
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int r = (tid >> 5) + 8 * u, l = tid & 31, i = i0 + r;
+    Cs[r][l] = (i < n && l < nb && !inK(i)) ? C[(size_t)i * GB + l] : 0.0f;
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = (tid >> 5) + 8 * u, c = tid & 31;
+    D[r][c] = (r < nb && c < nb) ? R[(size_t)r * n + k0 + c] : (r == c ? 1.0f : 0.0f);
   }
   __syncthreads();
   block_invert(D, rowk, colk);
-  if (blockIdx.x == 0)
-    for (int q = tid; q < GB * GB; q += 256) P[q] = D[q / GB][q % GB];
-  const int j0 = blockIdx.x * GT;
-  for (int q = tid; q < GB * GT; q += 256) {
-    const int l = q / GT, c = q % GT, j = j0 + c;
-    R[l][c] = (l < nb && j < n) ? A[(size_t)(k0 + l) * n + j] : 0.0f;
-  }
+#pragma unroll
+  for (int u = 0; u < 8; ++u) Bs[bl][bc + 8 * u] = rv[u];
   __syncthreads();
-  for (int q = tid; q < GB * GT; q += 256) {
-    const int l = q / GT, c = q % GT, j = j0 + c;
-    if (l >= nb || j >= n || (j >= k0 && j < k0 + nb)) continue;
-    float s = 0.0f;
+  float b[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) b[u] = 0.0f;
 #pragma unroll 8
-    for (int m = 0; m < GB; ++m) s += D[l][m] * R[m][c];
-    A[(size_t)(k0 + l) * n + j] = s;
-  }
-  for (int q = tid; q < GT * GB; q += 256) {
-    const int r = q / GB, l = q % GB, i = j0 + r;
-    if (i >= n) continue;
-    C[(size_t)i * GB + l] = (l < nb && !(i >= k0 && i < k0 + nb)) ? A[(size_t)i * n + k0 + l] : 0.0f;
-  }
-}
-
-// Rest of the step, one GT x GT tile per CTA:
-//   i, j not in K:  A_ij <- A_ij - sum_l C_il A_Kj,l   (row block already new)
-//   i not in K, j in K:  A_iK <- -C_i P
-//   i, j in K:  A_KK <- P
-__global__ void __launch_bounds__(256) k_gj_update(float *A, int n, int k0, int nb, const float *P,
-                                                   const float *C) {
-  __shared__ float Cs[GT][GB + 1];
-  __shared__ float Bs[GB][GT + 1];
-  const int nt = (n + GT - 1) / GT;
-  const int ti = blockIdx.x / nt, tj = blockIdx.x % nt;
-  const int i0 = ti * GT, j0 = tj * GT, tid = threadIdx.x;
-  auto inK = [&](int x) { return x >= k0 && x < k0 + nb; };
-  for (int q = tid; q < GT * GB; q += 256) {
-    const int r = q / GB, l = q % GB, i = i0 + r;
-    Cs[r][l] = (i < n) ? C[(size_t)i * GB + l] : 0.0f;
-  }
-  for (int q = tid; q < GB * GT; q += 256) {
-    const int l = q / GT, c = q % GT, j = j0 + c;
-    float b = 0.0f;
-    if (j < n && l < nb) b = inK(j) ? P[l * GB + (j - k0)] : A[(size_t)(k0 + l) * n + j];
-    Bs[l][c] = b;
+  for (int m = 0; m < GB; ++m) {
+    const float p = D[bl][m];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) b[u] += p * Bs[m][bc + 8 * u];
   }
   __syncthreads();
-  const int tx = tid % 16, ty = tid / 16;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int j = j0 + bc + 8 * u;
+    Bs[bl][bc + 8 * u] = inK(j) ? D[bl][j - k0] : b[u];
+  }
+  __syncthreads();
   float acc[4][4] = {};
 #pragma unroll 8
   for (int l = 0; l < GB; ++l) {
-    float a[4], b[4];
+    float c[4], w[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      a[u] = Cs[ty + 16 * u][l];
-      b[u] = Bs[l][tx + 16 * u];
+      c[u] = Cs[ty + 16 * u][l];
+      w[u] = Bs[l][tx + 16 * u];
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u)
 #pragma unroll
-      for (int v = 0; v < 4; ++v) acc[u][v] += a[u] * b[v];
+      for (int v = 0; v < 4; ++v) acc[u][v] += c[u] * w[v];
   }
+  const int k1 = k0 + GB;   // next block
 #pragma unroll
   for (int u = 0; u < 4; ++u)
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
       const int i = i0 + ty + 16 * u, j = j0 + tx + 16 * v;
       if (i >= n || j >= n) continue;
-      float *a = A + (size_t)i * n + j;
-      if (inK(i)) {
-        if (inK(j)) *a = P[(i - k0) * GB + (j - k0)];
-      } else if (inK(j)) {
-        *a = -acc[u][v];
-      } else {
-        *a -= acc[u][v];
-      }
+      const float x = inK(i) ? Bs[i - k0][tx + 16 * v] : a[u][v] - acc[u][v];
+      A[(size_t)i * n + j] = x;
+      if (i >= k1 && i < k1 + GB) Rn[(size_t)(i - k1) * n + j] = x;
+      if (j >= k1 && j < k1 + GB) Cn[(size_t)i * GB + (j - k1)] = x;
     }
 }
 
@@ -199,40 +221,45 @@ __global__ void k_ir_correct(const float *Ainv, int n, const double *dsc, const 
   if (lane == 0) x[row] += dsc[row] * (double)s;
 }
 
-// r = g - S~ x (FP64, one warp per row); rs = D r in FP32; scal[0] += |r|^2
+// r = g - S~ x (FP64, one warp per row); rs = D r in FP32; scal[0] += |r|^2.
+// The CTA that finishes last (flag[3] counts them) tests convergence,
+// |r|^2 <= eps^2 |g|^2 -> flag[0] = 1; scal[2] keeps the last |r|^2.
 __global__ void k_ir_residual(const double *S, int n, const double *g, const double *x,
-                              const double *dsc, double *r, float *rs, double *scal,
-                              const int *flag) {
+                              const double *dsc, double *r, float *rs, double *scal, int *flag,
+                              double eps2) {
   if (flag[0] | flag[1]) return;
   const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (row >= n) return;
-  const double *a = S + (size_t)row * n;
-  double s0 = 0.0, s1 = 0.0;
-  int j = lane;
-  for (; j + 32 < n; j += 64) {
-    s0 += a[j] * x[j];
-    s1 += a[j + 32] * x[j + 32];
+  if (row < n) {
+    const double *a = S + (size_t)row * n;
+    double s0 = 0.0, s1 = 0.0;
+    int j = lane;
+    for (; j + 32 < n; j += 64) {
+      s0 += a[j] * x[j];
+      s1 += a[j + 32] * x[j + 32];
+    }
+    if (j < n) s0 += a[j] * x[j];
+    double s = s0 + s1;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) {
+      const double v = g[row] - s;
+      r[row] = v;
+      rs[row] = (float)(dsc[row] * v);
+      atomicAdd(scal, v * v);
+      __threadfence();
+    }
   }
-  if (j < n) s0 += a[j] * x[j];
-  double s = s0 + s1;
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) {
-    const double v = g[row] - s;
-    r[row] = v;
-    rs[row] = (float)(dsc[row] * v);
-    atomicAdd(scal, v * v);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(flag + 3, 1) == (int)gridDim.x - 1) {
+      flag[3] = 0;
+      const double rr = atomicAdd(scal, 0.0);
+      scal[0] = 0.0;
+      scal[2] = rr;
+      flag[2] += 1;
+      if (rr <= eps2 * scal[1]) flag[0] = 1;
+    }
   }
-}
-
-// convergence: |r|^2 <= eps^2 |g|^2 -> flag[0] = 1; scal[2] keeps the last |r|^2
-__global__ void k_ir_check(double *scal, int *flag, double eps2) {
-  if (flag[0] | flag[1]) return;
-  const double rr = scal[0];
-  scal[0] = 0.0;
-  scal[2] = rr;
-  flag[2] += 1;
-  if (!(rr <= eps2 * scal[1])) return;
-  flag[0] = 1;
 }
 
 void ir_sequence(const SrWork &w, int max_iter, double eps, cudaStream_t st) {
@@ -240,26 +267,27 @@ void ir_sequence(const SrWork &w, int max_iter, double eps, cudaStream_t st) {
   cudaMemsetAsync(w.irflag, 0, sizeof(int) * 4, st);
   k_ir_diag<<<(n + 255) / 256, 256, 0, st>>>(w.S, n, w.dsc, w.irflag);
   const size_t n2 = (size_t)n * n;
-  k_ir_scale<<<(unsigned)((n2 + 255) / 256), 256, 0, st>>>(w.S, n, w.dsc, w.S32);
+  // the pivot block's rows and columns, alternating between two buffers
+  float *R[2] = {w.gjR, w.gjR + (size_t)GB * n}, *C[2] = {w.gjC, w.gjC + (size_t)GB * n};
+  k_ir_scale<<<(unsigned)((n2 + 255) / 256), 256, 0, st>>>(w.S, n, w.dsc, w.S32, R[0], C[0]);
   const int nt = (n + GT - 1) / GT;
-  for (int k0 = 0; k0 < n; k0 += GB) {
+  for (int k0 = 0, q = 0; k0 < n; k0 += GB, q ^= 1) {
     const int nb = n - k0 < GB ? n - k0 : GB;
-    k_gj_row<<<nt, 256, 0, st>>>(w.S32, n, k0, nb, w.gjP, w.gjC);
-    k_gj_update<<<nt * nt, 256, 0, st>>>(w.S32, n, k0, nb, w.gjP, w.gjC);
+    k_gj_step<<<nt * nt, 256, 0, st>>>(w.S32, n, k0, nb, R[q], C[q], R[q ^ 1], C[q ^ 1]);
   }
   k_ir_init<<<1, 256, 0, st>>>(w.g, n, w.dsc, w.x, w.r, w.rs32, w.scal, w.irflag);
   const int wb = (int)(((size_t)n * 32 + 255) / 256);
   for (int it = 0; it < max_iter; ++it) {
     k_ir_correct<<<wb, 256, 0, st>>>(w.S32, n, w.dsc, w.rs32, w.x, w.irflag);
-    k_ir_residual<<<wb, 256, 0, st>>>(w.S, n, w.g, w.x, w.dsc, w.r, w.rs32, w.scal, w.irflag);
-    k_ir_check<<<1, 1, 0, st>>>(w.scal, w.irflag, eps * eps);
+    k_ir_residual<<<wb, 256, 0, st>>>(w.S, n, w.g, w.x, w.dsc, w.r, w.rs32, w.scal, w.irflag,
+                                      eps * eps);
   }
 }
 
 }  // namespace
 
 long long vmc_sr_ir_launches(int n, int max_iter) {
-  return 3 + 2LL * ((n + GB - 1) / GB) + 3LL * max_iter;
+  return 3 + (n + GB - 1) / GB + 2LL * max_iter;
 }
 
 // Launch the refinement (the captured graph, made on first use).  Returns 0
