@@ -412,7 +412,7 @@ struct GJSteps {
   double val[ST_WARPS];
   double amax[ST_WARPS];
   unsigned long long ckey[2][ST_WARPS];   // per-warp pivot candidates (|a| bits) ...
-  int cidx[2][ST_WARPS];                  // ... and their rows, double-buffered by step
+  int cidx[2][ST_WARPS];                  // ... and their signed_row()s, double-buffered by step
   int bad;
   int sign;
   double logdet;
@@ -429,6 +429,11 @@ struct GJSteps {
 __device__ __forceinline__ unsigned long long pivot_key(double a) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFull;
   return b > 0x7FF0000000000000ull ? 0ull : b + 1ull;
+}
+
+// a candidate's row with the sign of its entry in the lowest bit
+__device__ __forceinline__ int signed_row(int i, double a) {
+  return 2 * i + (__double2hiint(a) < 0 ? 1 : 0);
 }
 
 // warp-wide largest key (ties: lowest row); lane 0 records it in slot buf
@@ -462,12 +467,13 @@ __device__ __forceinline__ void gj_steps(double *A, int lda, int N, int *perm, G
   // candidates of column 0
   {
     unsigned long long key = 0ull;
-    int row = N;
+    int row = 2 * N;
     for (int i = tid; i < N; i += nth) {
-      const unsigned long long kk = pivot_key(A[(size_t)i * lda]);
+      const double v = A[(size_t)i * lda];
+      const unsigned long long kk = pivot_key(v);
       if (kk > key) {
         key = kk;
-        row = i;
+        row = signed_row(i, v);
       }
     }
     pivot_candidates(key, row, g, 0);
@@ -491,21 +497,25 @@ __device__ __forceinline__ void gj_steps(double *A, int lda, int N, int *perm, G
     // copy of column k+1 (the two touch disjoint columns).
     if (tid < 64) {
       unsigned long long bk = g.ckey[buf][0];
-      int p = g.cidx[buf][0];
+      int row = g.cidx[buf][0];
       for (int q = 1; q < nwarp; ++q) {
         const unsigned long long kq = g.ckey[buf][q];
         const int iq = g.cidx[buf][q];
-        if (kq > bk || (kq == bk && iq < p)) {
+        if (kq > bk || (kq == bk && iq < row)) {
           bk = kq;
-          p = iq;
+          row = iq;
         }
       }
+      const int p = row >> 1;
       const int lane = tid & 31;
-      if (bk <= 1ull || p >= N) {   // zero (key 1) or no finite entry: singular
+      const bool singular = bk <= 1ull || p >= N;   // zero (key 1) or no finite entry
+      // the pivot from its candidate, not from A: warp 0 writes column k while
+      // warp 1 may not have started
+      const double piv = __longlong_as_double((long long)((bk - 1ull) | (unsigned long long)(row & 1) << 63));
+      const double ipiv = __drcp_rn(piv);
+      if (singular) {
         if (tid == 0) g.bad = 1;
       } else if (tid < 32) {
-        const double piv = A[(size_t)p * lda + k];
-        const double ipiv = __drcp_rn(piv);
         if (tid == 0) {
           perm[k] = p;
           g.ipiv = ipiv;
@@ -522,7 +532,6 @@ __device__ __forceinline__ void gj_steps(double *A, int lda, int N, int *perm, G
         // leaves it through the update)
         for (int i = lane; i < N; i += 32) A[(size_t)i * lda + k] = (i == k) ? ipiv : g.colk[i];
       } else {
-        const double ipiv = __drcp_rn(A[(size_t)p * lda + k]);
         for (int c = lane; c < N; c += 32) {
           if (c == k) {
             g.rowk[c] = 0.0;
@@ -547,13 +556,13 @@ __device__ __forceinline__ void gj_steps(double *A, int lda, int N, int *perm, G
     // no barrier of its own
     if (k1 < N) {
       unsigned long long key = 0ull;
-      int row = N;
+      int row = 2 * N;
       for (int i = tid; i < N; i += nth) {
         const double v = fma(g.colk[i], g.rowk[k1], g.coln[i]);
         const unsigned long long kk = pivot_key(v);
         const bool t = (i >= k1) & (kk > key);
         key = t ? kk : key;
-        row = t ? i : row;
+        row = t ? signed_row(i, v) : row;
       }
       pivot_candidates(key, row, g, buf ^ 1);
     }
