@@ -1378,8 +1378,8 @@ int vmc_measure_corr(vmc_ctx *c, int32_t system, double *corr, double *ms) {
   CK(upload_sysdesc(c));
   const int prec = c->precision == VMC_FP64 ? 0 : 1;
   // the pair-correlation kernel reads the FP32 words only
-  const size_t smem_corr = vmc_walker_smem(prec, s.N, s.Ns, s.Np, s.dev.n_hidden, 0, nullptr, 0);
-  const int grid = vmc_corr_grid(prec, smem_corr, s.W, s.Ns);
+  CorrShape shape;
+  CKC(vmc_corr_shape(prec, s.N, s.Ns, s.W, &shape));
   const size_t ns2 = (size_t)s.Ns * s.Ns;
   const size_t part_b = 3 * ns2 * sizeof(double);
   const size_t cnt_b = (4 * ns2 * sizeof(int) + 255) / 256 * 256;
@@ -1409,9 +1409,9 @@ int vmc_measure_corr(vmc_ctx *c, int32_t system, double *corr, double *ms) {
       }
   int rc = VMC_OK;
   if ((ms && cudaEventRecord(ev[0], c->st)) || cudaMemsetAsync(part, 0, part_b, c->st) ||
-      vmc_launch_corr_occ(c->d_sys, system, s.Ns, cnt, c->st, &c->n_launch) ||
+      vmc_launch_corr_occ(c->d_sys, system, s.Ns, s.W, cnt, c->st, &c->n_launch) ||
       (ms && cudaEventRecord(ev[1], c->st)) ||
-      vmc_launch_corr(c->d_sys, system, prec, grid, part, smem_corr, c->st, &c->n_launch) ||
+      vmc_launch_corr(c->d_sys, system, prec, s.N, shape, part, c->st, &c->n_launch) ||
       (ms && cudaEventRecord(ev[2], c->st)) ||
       vmc_launch_corr_reduce(part, 1, cnt, s.Ns, s.W, s.dev.lsite, out, c->st, &c->n_launch) ||
       (ms && cudaEventRecord(ev[3], c->st)) ||

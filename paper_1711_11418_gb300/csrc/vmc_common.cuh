@@ -136,20 +136,26 @@ cudaError_t vmc_launch_eval_ratios(const SysDev *d_sys, int sys, int walker,
                                    int precision, int n_moves, const int *d_moves,
                                    double *d_out, size_t smem, cudaStream_t st,
                                    long long *n_launch);
-// Pair correlations (measurement mode): CTA count of k_corr (occupancy x SMs,
-// at most W), the ratio kernel (adds into FP64 planes [3][Ns][Ns]), the
-// occupation-count kernel (int [4][Ns][Ns]) and the reduction into
-// double [6][Ns][Ns].
-int vmc_corr_grid(int precision, size_t smem, int W, int Ns);
-cudaError_t vmc_launch_corr(const SysDev *d_sys, int sys, int precision, int grid,
-                            double *part, size_t smem, cudaStream_t st, long long *n_launch);
-cudaError_t vmc_launch_corr_occ(const SysDev *d_sys, int sys, int Ns, int *cnt,
+// Pair correlations (measurement mode): the launch shape of k_corr for one
+// system, the ratio kernel (adds into FP64 planes [3][Ns][Ns], kind 4's
+// transposed), the occupation-count kernel (int [4][Ns][Ns]) and the reduction
+// into double [6][Ns][Ns].
+struct CorrShape {
+  int grid;      // CTAs: resident ones, at most W
+  int rows;      // rows of G_up held in shared memory
+  size_t smem;   // dynamic shared memory in bytes
+};
+cudaError_t vmc_corr_shape(int precision, int N, int Ns, int W, CorrShape *out);
+cudaError_t vmc_launch_corr(const SysDev *d_sys, int sys, int precision, int N,
+                            const CorrShape &shape, double *part, cudaStream_t st,
+                            long long *n_launch);
+cudaError_t vmc_launch_corr_occ(const SysDev *d_sys, int sys, int Ns, int W, int *cnt,
                                 cudaStream_t st, long long *n_launch);
 cudaError_t vmc_launch_corr_reduce(const double *part, int n_part, const int *cnt, int Ns,
                                    int W, const signed char *lsite, double *out, cudaStream_t st,
                                    long long *n_launch);
 // with_lo: the mixed form's sweep keeps the low words of its double-float
-// M^-1 in shared memory as well (the pair-correlation kernel does not).
+// M^-1 in shared memory as well.
 size_t vmc_walker_smem(int precision, int N, int Ns, int Np, int H, int kd, int *acc_len,
                        int with_lo);
 size_t vmc_init_smem(int N, int Ns, int form);

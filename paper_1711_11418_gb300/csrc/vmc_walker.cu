@@ -2365,251 +2365,6 @@ __global__ void __launch_bounds__(NT) k_eval_ratios(const SysDev *systems, int s
   }
 }
 
-// ---------------------------------------------------------------------------
-// Pair correlations of the current configurations (measurement mode,
-// Sec. 2.2.3; local estimators of Eq. MC, A acting on the ket |x>).
-//
-// Off-diagonal kinds, per walker, from Green-function ratios of its M^-1 = B:
-//   G_up[b, k] = sum_l f(b, r_l,dn) B_lk      (up electron k hops to b)
-//   G_dn[a, m] = sum_k f(r_k,up, a) B_mk      (down electron m hops to a)
-//   T[b, a]    = sum_k G_up[b, k] f(r_k,up, a)
-// and, for the spin swap of up electron n on a with down electron m on b
-// (both sites singly occupied; det of M with row n and column m replaced),
-//   det M'/det M = G_up[b, n] G_dn[a, m] - B_mn (T[b, a] - f(b, a)).
-// One pass over the sites b: G_up[b, :] (N^2); the down-occupied sites are
-// collected in groups of CORR_G, and for a group G_dn[:, m] and T[b, :] of
-// all its sites are formed together (2 N Ns each), so every gathered
-// f(r_k,up, a) serves 2 CORR_G products: Ns N^2 + 2 N_dn N Ns per
-// configuration for all Ns^2 pairs.
-//   kind 0 (c^dag_{b up} c_{j up}): up electron on j hops to b,
-//          G_up[b, k] x P_G P_J ratio;
-//   kind 1 (c^dag_{a dn} c_{b dn}): down electron on b hops to a,
-//          G_dn[a, m] x P_G P_J ratio;
-//   kind 4 (S^+_b S^-_a): the swap above, with the fermion sign -1 of
-//          S^+S^- in the labelled basis (P_G, P_J unchanged).
-// Each CTA takes walkers blockIdx.x, blockIdx.x + gridDim.x, ... in turn and
-// adds their values to one FP64 plane triple part[3][Ns][Ns] (diagonal
-// entries stay 0) by atomic adds without return, so the 24 Ns^2 bytes stay
-// in L2 and no thread waits on them; the order of the additions, and so the
-// last bit of a sum, varies between runs.
-// ---------------------------------------------------------------------------
-// Down-occupied sites whose second product is formed together (their G_up
-// rows wait in vector slots 1..CORR_G of shared memory).
-constexpr int CORR_G = 4;
-
-template <typename T>
-__global__ void __launch_bounds__(NT) k_corr(const SysDev *systems, int sys, double *part) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ SysDev S;
-  load_sys(&S, systems + sys);
-  const int N = S.N, Ns = S.Ns, Ne = S.Ne, ldm = S.ldm, tid = threadIdx.x;
-  WSmem<T> sm;
-  walker_layout<T>(N, Ns, S.acc_len, S.n_hidden, 0, false, smem_raw, &sm);
-  T *fb = sm.vec;                    // slot 0: f(b, r_l,dn), l < N
-  const T *F = ftab<T>(S);
-  const size_t ns2 = (size_t)Ns * Ns;
-  double *P0 = part;
-  double *P1 = P0 + ns2;
-  double *P4 = P1 + ns2;
-  const size_t nb = minv_bytes(N, ldm, sizeof(T));
-  for (int w = blockIdx.x; w < S.W; w += gridDim.x) {
-    const T *src = (const T *)((const unsigned char *)S.minv + (size_t)w * nb);
-    for (int k = tid; k < N * ldm; k += NT) sm.minv[k] = src[k];
-    for (int k = tid; k < Ne; k += NT) sm.ele[k] = S.ele[(size_t)w * Ne + k];
-    for (int k = tid; k < 2 * Ns; k += NT) sm.occ[k] = S.occ[(size_t)w * 2 * Ns + k];
-    for (int k = tid; k < Ns; k += NT) sm.jf[k] = ((const T *)S.jf)[(size_t)w * Ns + k];
-    __syncthreads();
-    // pending group: sites gb[q] with down electron gm[q], G_up row in slot 1 + q
-    int ng = 0;
-    int gb[CORR_G], gm[CORR_G];
-#pragma unroll
-    for (int q = 0; q < CORR_G; ++q) gb[q] = gm[q] = 0;
-    // G_up[b, :] = f(b, r_dn)^T M^-1 for four sites b at a time: the rows
-    // f(b, r_l,dn) in vector slots 0, 5, 6, 7, thread k the column k, one
-    // shared load of M^-1 per four multiply-adds; the rows of down-occupied
-    // sites go to the group's slots 1..CORR_G.
-    T *fbs[4] = {fb, sm.vec + 5 * VMC_MAX_N, sm.vec + 6 * VMC_MAX_N, sm.vec + 7 * VMC_MAX_N};
-    for (int b0 = 0; b0 < Ns; b0 += 4) {
-      const int nbk = (Ns - b0 < 4) ? Ns - b0 : 4;
-      if (tid < N) {
-        const int el = sm.ele[N + tid];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          fbs[u][tid] = (u < nbk) ? F[(size_t)(b0 + u) * Ns + el] : (T)0;
-      }
-      __syncthreads();
-      T g4[4] = {(T)0, (T)0, (T)0, (T)0};
-      if (tid < N) {
-        int l = 0;
-        for (; l + 4 <= N; l += 4) {
-          const T m0 = sm.minv[l * ldm + tid], m1 = sm.minv[(l + 1) * ldm + tid];
-          const T m2 = sm.minv[(l + 2) * ldm + tid], m3 = sm.minv[(l + 3) * ldm + tid];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            T x0, x1, x2, x3;
-            ld4(fbs[u] + l, x0, x1, x2, x3);
-            g4[u] += x0 * m0;
-            g4[u] += x1 * m1;
-            g4[u] += x2 * m2;
-            g4[u] += x3 * m3;
-          }
-        }
-        for (; l < N; ++l) {
-          const T m0 = sm.minv[l * ldm + tid];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) g4[u] += fbs[u][l] * m0;
-        }
-      }
-      __syncthreads();   // the block's rows are read; slots 0, 5..7 free
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (u >= nbk) break;
-        const int b = b0 + u;
-        const bool b_up = sm.occ[b] >= 0, b_dn = sm.occ[Ns + b] >= 0;
-        // kind 0 at (b, r_k,up)
-        if (tid < N && !b_up && !(S.local_spin && b_dn)) {
-          const int j = sm.ele[tid];
-          const T c = corr_factor<T>(corr_hop<T>(S, sm.occ, sm.jf, 0, j, b));
-          atomicAdd(&P0[(size_t)b * Ns + j], (double)(g4[u] * c));
-        }
-        if (b_dn) {
-          if (tid < N) sm.vec[(size_t)(1 + ng) * VMC_MAX_N + tid] = g4[u];
-  #pragma unroll
-          for (int q = 0; q < CORR_G; ++q)
-            if (q == ng) {
-              gb[q] = b;
-              gm[q] = sm.occ[Ns + b] - N;
-            }
-          ++ng;
-        }
-        if (ng == CORR_G || (b == Ns - 1 && ng > 0)) {
-          __syncthreads();   // the group's G_up rows are in place
-          // G_dn[a, m] and T[b, a] of the group's sites, two sites a per
-          // thread: each f(r_k,up, a) feeds 2 x CORR_G pairs of products.
-          const T *Bq[CORR_G], *Gq[CORR_G];
-  #pragma unroll
-          for (int q = 0; q < CORR_G; ++q) {
-            Bq[q] = sm.minv + (size_t)gm[q] * ldm;       // unused slots: a valid row
-            Gq[q] = sm.vec + (size_t)(1 + q) * VMC_MAX_N;
-          }
-          for (int a0 = tid; a0 < Ns; a0 += 2 * NT) {
-            const int a1 = a0 + NT < Ns ? a0 + NT : a0;
-            T d0[CORR_G], t0[CORR_G], d1[CORR_G], t1[CORR_G];
-  #pragma unroll
-            for (int q = 0; q < CORR_G; ++q) d0[q] = t0[q] = d1[q] = t1[q] = (T)0;
-            for (int k = 0; k < N; ++k) {
-              const T *Fk = F + (size_t)sm.ele[k] * Ns;
-              const T f0 = Fk[a0], f1 = Fk[a1];
-  #pragma unroll
-              for (int q = 0; q < CORR_G; ++q) {
-                const T bk = Bq[q][k], gk = Gq[q][k];
-                d0[q] += bk * f0;
-                t0[q] += gk * f0;
-                d1[q] += bk * f1;
-                t1[q] += gk * f1;
-              }
-            }
-  #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const int a = h ? a1 : a0;
-              if (h && a1 == a0) break;
-              const bool a_up = sm.occ[a] >= 0, a_dn = sm.occ[Ns + a] >= 0;
-  #pragma unroll
-              for (int q = 0; q < CORR_G; ++q) {
-                if (q >= ng) break;
-                const int bq = gb[q];
-                if (a == bq) continue;
-                const T accD = h ? d1[q] : d0[q], accT = h ? t1[q] : t0[q];
-                // kind 1 at (a, bq): down electron gm[q] hops bq -> a
-                if (!a_dn && !(S.local_spin && a_up)) {
-                  const T c = corr_factor<T>(corr_hop<T>(S, sm.occ, sm.jf, 1, bq, a));
-                  atomicAdd(&P1[(size_t)a * Ns + bq], (double)(accD * c));
-                }
-                // kind 4 at (bq, a): spin swap with up electron n on a
-                if (a_up && !a_dn && sm.occ[bq] < 0) {
-                  const int n = sm.occ[a];
-                  const T r = Gq[q][n] * accD - Bq[q][n] * (accT - F[(size_t)bq * Ns + a]);
-                  atomicAdd(&P4[(size_t)bq * Ns + a], -(double)r);
-                }
-              }
-            }
-          }
-          ng = 0;
-          __syncthreads();   // the group's slots are written again
-        }
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// Occupation products summed over the walkers of one system, exactly in
-// integers: cnt[c][i][j] = sum_w x_i y_j with (x, y) = (n_up, n_up),
-// (n_up, n_dn), (n_dn, n_up), (n_dn, n_dn) for c = 0..3.  These give every
-// diagonal estimator (n_i n_j, S^z_i S^z_j and the i = j terms of kinds 0, 1,
-// 4, 5).  One thread per (i, j) of a 16 x 16 tile.
-__global__ void k_corr_occ(const SysDev *systems, int sys, int *cnt) {
-  const SysDev &S = systems[sys];
-  const int Ns = S.Ns;
-  const int i = blockIdx.y * 16 + threadIdx.y, j = blockIdx.x * 16 + threadIdx.x;
-  if (i >= Ns || j >= Ns) return;
-  int uu = 0, ud = 0, du = 0, dd = 0;
-  for (int w = 0; w < S.W; ++w) {
-    const int *o = S.occ + (size_t)w * 2 * Ns;
-    const int ui = o[i] >= 0, di = o[Ns + i] >= 0, uj = o[j] >= 0, dj = o[Ns + j] >= 0;
-    uu += ui & uj;
-    ud += ui & dj;
-    du += di & uj;
-    dd += di & dj;
-  }
-  const size_t ns2 = (size_t)Ns * Ns, q = (size_t)i * Ns + j;
-  cnt[q] = uu;
-  cnt[ns2 + q] = ud;
-  cnt[2 * ns2 + q] = du;
-  cnt[3 * ns2 + q] = dd;
-}
-
-// out[kind][i][j] = walker mean of the local estimators (kinds 0..5 of the
-// header): the ratio planes (n_part sets, summed in order) and the integer
-// counts, scaled.  With a local_site mask (Kondo local spins: exactly one
-// electron each) a hop c^dag_i c_j with i != j into or out of a marked site
-// leaves the constrained space, where psi = 0: those entries of kinds 0 and 1
-// are 0.  Spin swaps keep every site's occupation and are kept.
-__global__ void k_corr_reduce(const double *part, int n_part, const int *cnt, int Ns, int W,
-                              const signed char *lsite, double *out) {
-  const size_t ns2 = (size_t)Ns * Ns;
-  const double inv = 1.0 / (double)W;
-  for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < ns2;
-       q += (size_t)gridDim.x * blockDim.x) {
-    const int i = (int)(q / Ns), j = (int)(q % Ns);
-    const size_t qt = (size_t)j * Ns + i;
-    double g0 = 0.0, g1 = 0.0, s4 = 0.0, s4t = 0.0;
-    for (int b = 0; b < n_part; ++b) {
-      const double *P = part + (size_t)b * 3 * ns2;
-      g0 += P[q];
-      g1 += P[ns2 + q];
-      s4 += P[2 * ns2 + q];
-      s4t += P[2 * ns2 + qt];
-    }
-    const double uu = cnt[q], ud = cnt[ns2 + q], du = cnt[2 * ns2 + q], dd = cnt[3 * ns2 + q];
-    const double szsz = 0.25 * (uu - ud - du + dd);
-    double d0 = 0.0, d1 = 0.0, d4 = 0.0, d5 = 0.0;
-    if (i == j) {   // n_up, n_dn, n_up (1 - n_dn), (n_up + n_dn - 2 n_up n_dn) / 2
-      d0 = uu;
-      d1 = dd;
-      d4 = uu - ud;
-      d5 = 0.5 * (uu - ud + dd - du);
-    }
-    if (lsite && i != j && (lsite[i] | lsite[j])) g0 = g1 = 0.0;
-    out[q] = (g0 + d0) * inv;
-    out[ns2 + q] = (g1 + d1) * inv;
-    out[2 * ns2 + q] = (uu + ud + du + dd) * inv;
-    out[3 * ns2 + q] = szsz * inv;
-    out[4 * ns2 + q] = (s4 + d4) * inv;
-    out[5 * ns2 + q] = (szsz + 0.5 * (s4 + s4t) + d5) * inv;
-  }
-}
-
 #endif  // VMC_SWEEP_V3_ONLY
 }  // namespace
 
@@ -2674,8 +2429,6 @@ cudaError_t vmc_walker_set_smem_limits(size_t s64, size_t s32, size_t sinit) {
   if ((e = cudaFuncSetAttribute(k_sample<float, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s32))) return e;
   if ((e = vmc_sample_set_smem_v3(s32))) return e;
   if ((e = cudaFuncSetAttribute(k_eval_ratios<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s32))) return e;
-  if ((e = cudaFuncSetAttribute(k_corr<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s64))) return e;
-  if ((e = cudaFuncSetAttribute(k_corr<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s32))) return e;
   for (int form : {VMC_INIT_BLOCKED, VMC_INIT_STEPS, VMC_INIT_DF})
     for (int prec = 0; prec < 2; ++prec)
       for (int nth : {NT, vmc_gj::MAX_THREADS})
@@ -2753,50 +2506,6 @@ cudaError_t vmc_launch_eval_ratios(const SysDev *d_sys, int sys, int walker, int
     k_eval_ratios<double><<<1, NT, smem, st>>>(d_sys, sys, walker, n_moves, d_moves, d_out);
   else
     k_eval_ratios<float><<<1, NT, smem, st>>>(d_sys, sys, walker, n_moves, d_moves, d_out);
-  ++*nl;
-  return cudaGetLastError();
-}
-
-int vmc_corr_grid(int precision, size_t smem, int W, int Ns) {
-  int dev = 0, nsm = 0, per = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (precision == 0)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_corr<double>, NT, smem);
-  else
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_corr<float>, NT, smem);
-  if (per < 1) per = 1;
-  long long grid = (long long)nsm * per;
-  if (grid > W) grid = W;
-  if (grid < 1) grid = 1;
-  return (int)grid;
-}
-
-cudaError_t vmc_launch_corr(const SysDev *d_sys, int sys, int precision, int grid, double *part,
-                            size_t smem, cudaStream_t st, long long *nl) {
-  if (precision == 0)
-    k_corr<double><<<grid, NT, smem, st>>>(d_sys, sys, part);
-  else
-    k_corr<float><<<grid, NT, smem, st>>>(d_sys, sys, part);
-  ++*nl;
-  return cudaGetLastError();
-}
-
-cudaError_t vmc_launch_corr_occ(const SysDev *d_sys, int sys, int Ns, int *cnt, cudaStream_t st,
-                                long long *nl) {
-  const dim3 blk(16, 16), grd((Ns + 15) / 16, (Ns + 15) / 16);
-  k_corr_occ<<<grd, blk, 0, st>>>(d_sys, sys, cnt);
-  ++*nl;
-  return cudaGetLastError();
-}
-
-cudaError_t vmc_launch_corr_reduce(const double *part, int n_part, const int *cnt, int Ns, int W,
-                                   const signed char *lsite, double *out, cudaStream_t st,
-                                   long long *nl) {
-  const size_t ns2 = (size_t)Ns * Ns;
-  const size_t blocks = (ns2 + 255) / 256;
-  const int grid = (int)(blocks < 4096 ? blocks : 4096);
-  k_corr_reduce<<<grid, 256, 0, st>>>(part, n_part, cnt, Ns, W, lsite, out);
   ++*nl;
   return cudaGetLastError();
 }
