@@ -380,7 +380,8 @@ __device__ __forceinline__ double gj_inverse_at(const double *A, int N, int k, i
 // ---------------------------------------------------------------------------
 // The elimination step by step, every multiply-add in FP64.  The blocked form
 // above differs from it in the last bits (about 1e-14 of the inverse, at no
-// larger error).  Two users of the inverse turn last bits into visible
+// larger error).  It takes the matrices close to singular; and two users of the
+// inverse turn last bits into visible
 // differences of a trajectory and keep this form: the mixed form's projected
 // state, whose FP32 inverses have no low words and whose ratios are sums over
 // the operations that cancel, and the mixed form of models with exchange
@@ -425,6 +426,22 @@ struct GJSteps {
   double pminw[ST_WARPS];
 };
 
+// A matrix the blocked form finds close to singular (max|M^-1| times the
+// largest pivot above this, or no pivot at all) is eliminated again step by
+// step.  The two forms' inverses differ by about 1e-16 of that product; the
+// spin swap of the pair correlations, a difference of products of two entries
+// that nearly cancel, multiplies it by the product's square, and one walker in
+// thousands then decides the mean.  4096 placements at N = 112, mixed form: the
+// correlations differ from those of the step-by-step inverses by up to 0.8 of
+// their size with the blocked form alone, by 2e-5 with 3000 here (5e-7 with
+// 1000); k_init takes 5.1, 5.9 and 6.2 ms.  About one random placement in 270
+// is above.
+constexpr double GJ_BLOCKED_COND = 3e3;
+// Where the second elimination keeps GJSteps: in the staged digits' space,
+// behind the part that its longer rows (odd stride) take.
+constexpr size_t GJ_REDO_OFFSET = sizeof(double) * VMC_MAX_N;
+static_assert(GJ_REDO_OFFSET + sizeof(GJSteps) <= GJ_STAGE_BYTES, "no room for the second elimination");
+
 // |a| as an ordered integer key; NaN below every number (never a pivot)
 __device__ __forceinline__ unsigned long long pivot_key(double a) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFull;
@@ -453,10 +470,10 @@ __device__ __forceinline__ void pivot_candidates(unsigned long long key, int row
   }
 }
 
-template <int NTH>   // threads of the CTA
+template <int NTH>   // threads of the CTA; 0: blockDim.x (at most 32 ST_WARPS)
 __device__ __forceinline__ void gj_steps(double *A, int lda, int N, int *perm, GJSteps &g) {
   const int tid = threadIdx.x;
-  constexpr int nth = NTH, nwarp = NTH / 32;
+  const int nth = NTH ? NTH : (int)blockDim.x, nwarp = nth / 32;
   if (tid == 0) {
     g.logdet = 0.0;
     g.sign = 1;

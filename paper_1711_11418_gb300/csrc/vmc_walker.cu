@@ -2168,7 +2168,7 @@ __global__ void __launch_bounds__(NTH, FORM == VMC_INIT_BLOCKED ? 2 : 0)
     constexpr bool ROWS = FORM != VMC_INIT_BLOCKED;
     unsigned char *scr = smem_raw + init_matrix_bytes(N, ROWS);
     int *ele = (int *)(scr + init_scratch_bytes(Ns, ROWS));   // Ne
-    int *perm = ele + Ne;                                     // N (not by panels)
+    int *perm = ele + Ne;                                     // N
     for (int k = tid; k < Ne; k += nth) ele[k] = S.ele[(size_t)w * Ne + k];
     __syncthreads();
     if constexpr (DF) {
@@ -2195,13 +2195,41 @@ __global__ void __launch_bounds__(NTH, FORM == VMC_INIT_BLOCKED ? 2 : 0)
       __syncthreads();
       vmc_gj::gj_invert(A, (uint32_t *)scr, N, gs);
     }
-    const int g_bad = gs.bad, g_sign = gs.sign;
-    const double g_logdet = gs.logdet, g_pmin = gs.pmin, g_pmax = gs.pmax;
+    int g_bad = gs.bad, g_sign = gs.sign;
+    double g_logdet = gs.logdet, g_pmin = gs.pmin, g_pmax = gs.pmax;
+    bool redone = false;   // by panels: close to singular, eliminated again step by step
+    if constexpr (FORM == VMC_INIT_BLOCKED) {
+      double amax = 0.0;
+      if (!g_bad)   // the inverse's entries, in the order they are stored
+        for (int r = tid >> 5; r < N; r += nth / 32)
+          for (int q = tid & 31; q < N; q += 32)
+            amax = fmax(amax, fabs(A[vmc_gj::gj_at(r, q, vmc_gj::gj_pad(N))]));
+      for (int o = 16; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+      if ((tid & 31) == 0) red_a[tid >> 5] = amax;
+      __syncthreads();
+      for (int q = 0; q < nth / 32; ++q) amax = fmax(amax, red_a[q]);
+      redone = g_bad || !(amax * g_pmax <= vmc_gj::GJ_BLOCKED_COND);
+      __syncthreads();
+      if (redone) {
+        vmc_gj::GJSteps &g2 = *(vmc_gj::GJSteps *)(scr + vmc_gj::GJ_REDO_OFFSET);
+        for (int q = tid; q < N * N; q += nth) {
+          const int n = q / N, m = q - n * N;
+          A[n * ldm + m] = S.f64[(size_t)ele[n] * Ns + ele[N + m]];
+        }
+        __syncthreads();
+        vmc_gj::gj_steps<0>(A, ldm, N, perm, g2);
+        g_bad = g2.bad;
+        g_sign = g2.sign;
+        g_logdet = g2.logdet;
+        g_pmin = g2.pmin;
+        g_pmax = g2.pmax;
+      }
+    }
     // the fresh inverse's entry (r, c) (FP64 value)
     auto fresh_at = [&](int r, int c) -> double {
       if constexpr (DF) return (double)Ah[r * ldm + c] + (double)Al[r * ldm + c];
       else if constexpr (FORM == VMC_INIT_STEPS) return A[r * ldm + c];
-      else return vmc_gj::gj_inverse_at(A, N, r, c, gs);
+      else return redone ? A[r * ldm + c] : vmc_gj::gj_inverse_at(A, N, r, c, gs);
     };
     const size_t nb = minv_bytes(N, ldm, sizeof(T));
     T *dst = (T *)((unsigned char *)S.minv + (size_t)w * nb);
