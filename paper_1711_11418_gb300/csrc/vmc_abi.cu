@@ -425,7 +425,7 @@ int sr_alloc(vmc_ctx *c, SysHost &s, bool need_S, bool need_ir = false) {
     CK(dalloc(c, &w.tf, sizeof(float) * rows_cap));
     CK(dalloc(c, &w.dpart, sizeof(double) * 512));
     const size_t nparts = (size_t)vmc_colreduce_parts(rows_cap, Np);
-    CK(dalloc(c, &w.part, sizeof(double) * nparts * Np));
+    CK(dalloc(c, &w.part, sizeof(double) * 2 * nparts * Np));
     s.sr_alloc = true;
   }
   if (need_S && !s.S_alloc) {
@@ -1048,7 +1048,7 @@ int vmc_get_sr_matrices(vmc_ctx *c, int32_t system, double shift_rel, double shi
   if (!s.rows) return VMC_ESTATE;
   CK(sr_alloc(c, s, S != nullptr));
   CKC(vmc_sr_means(s.sr, c->st, &c->n_launch));
-  CKC(vmc_sr_build_g(s.sr, c->st, &c->n_launch));
+  CKC(vmc_sr_build_g(s.sr, false, c->st, &c->n_launch));
   if (S) {
     CK(build_S(c, s, shift_rel, shift_abs));
     CKC(cudaMemcpyAsync(S, s.sr.S, sizeof(double) * (size_t)s.Np * s.Np, cudaMemcpyDeviceToHost, c->st));
@@ -1074,7 +1074,7 @@ int vmc_sr_step(vmc_ctx *c, int32_t system, const vmc_sr_opts *o, vmc_sr_report 
   s.s_kernel = VMC_S_KERNEL_NONE;
   TimedRegion tr(c, 2);
   CKC(vmc_sr_means(w, c->st, &c->n_launch));
-  CKC(vmc_sr_build_g(w, c->st, &c->n_launch));
+  CKC(vmc_sr_build_g(w, !ir && !chol && !dense, c->st, &c->n_launch));
   int iters = 0, fallback = 0;
   double rel_res = 0.0;
   if (ir) {
@@ -1096,7 +1096,6 @@ int vmc_sr_step(vmc_ctx *c, int32_t system, const vmc_sr_opts *o, vmc_sr_report 
     const double eps = o->cg_eps > 0.0 ? o->cg_eps : 1e-10;
     const int kmax = o->cg_kmax > 0 ? o->cg_kmax : 1000;
     if (dense) CK(build_S(c, s, o->shift_rel, o->shift_abs));
-    else CKC(vmc_sr_diag(w, c->st, &c->n_launch));
     const int rc = vmc_sr_cg_solve(w, o->shift_rel, o->shift_abs, eps, kmax, &iters, c->st,
                                    &c->n_launch, dense ? 1 : 0);
     if (rc) return rc;
@@ -1191,7 +1190,7 @@ int vmc_sr_step_all(vmc_ctx *c, const vmc_sr_opts *o, vmc_sr_report *reps) {
     SrWork &w = s.sr;
     cudaStream_t st = c->pool[si % np];
     CKC(vmc_sr_means(w, st, &c->n_launch));
-    CKC(vmc_sr_build_g(w, st, &c->n_launch));
+    CKC(vmc_sr_build_g(w, false, st, &c->n_launch));
     CK(build_S_launch(c, s, o->shift_rel, o->shift_abs, st));
     if (c->precision == VMC_MIXED)
       CKC(cudaMemcpyAsync(stg[si].tcstat, s.tc_status, sizeof(int), cudaMemcpyDeviceToHost, st));

@@ -211,7 +211,7 @@ struct SrWork {
   int *info;                   // device status
   double *dblk;                // [32*32] factored diagonal block in flight (Cholesky)
   double *dinv;                // [ceil(Np/32)*32*32] inverses of the diagonal blocks of L
-  double *part;                // column-reduction partials [vmc_colreduce_parts(rows, Np) * Np]
+  double *part;                // column-reduction partials [2 * vmc_colreduce_parts(rows, Np) * Np]
   float *vf, *tf;              // FP32 copies of the SR-CG vectors (mixed form) [Np], [rows]
   double *dpart;               // dot-product partials [512]
   void *chol_graph;            // cudaGraphExec_t of the Cholesky factor + solve (lazily built)
@@ -236,8 +236,8 @@ cudaError_t vmc_sr_syrk_digits(const SrWork &w, unsigned char *digits, int *emax
 cudaError_t vmc_sr_means(const SrWork &w, cudaStream_t st, long long *nl);
 cudaError_t vmc_sr_build_S(const SrWork &w, double shift_rel, double shift_abs,
                            cudaStream_t st, long long *nl);
-cudaError_t vmc_sr_build_g(const SrWork &w, cudaStream_t st, long long *nl);
-cudaError_t vmc_sr_diag(const SrWork &w, cudaStream_t st, long long *nl);
+// the force g and, with diag, the diagonal of S in the same pass
+cudaError_t vmc_sr_build_g(const SrWork &w, bool diag, cudaStream_t st, long long *nl);
 int vmc_sr_cholesky_solve(SrWork &w, cudaStream_t st, long long *nl);
 void vmc_sr_release(SrWork &w);
 int vmc_sr_ir_solve(SrWork &w, int max_iter, double eps, int *iters, double *rel_res,
