@@ -202,6 +202,31 @@ __device__ __forceinline__ T block_sum(T v, T *red, int &buf) {
   return s;
 }
 
+// FP64 sums of the first N threads' values (N <= VMC_MAX_N; the other threads
+// hold 0).  A warp's FP64 instruction takes 64 cycles of its SM quarter, so the
+// additions of zeros that the full butterfly makes are left out: lanes and
+// warps from N on.  Same result as block_sum.  With accept_hop's screening:
+// 200 sweeps of 64 walkers of an 8-site ring 2.43 -> 1.83 ms, 4 of 1024 walkers
+// at 8 x 8 (N = 32) 1.76 -> 1.32 ms.
+__device__ __forceinline__ double warp_sum_first(double v, int N) {
+  for (int o = (N >= 32) ? 16 : (1 << (32 - __clz(N - 1))) >> 1; o > 0; o >>= 1)
+    v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;   // lane 0's is the sum
+}
+__device__ __forceinline__ double block_sum_first(double v, int N, double *red, int &buf) {
+  const int warp = threadIdx.x >> 5, nw = (N + 31) >> 5;
+  if (warp < nw) {
+    v = warp_sum_first(v, N);
+    if ((threadIdx.x & 31) == 0) red[buf * 16 + warp] = v;
+  }
+  __syncthreads();
+  const double *r = red + buf * 16;
+  double s = r[0];
+  for (int k = 1; k < nw; ++k) s += r[k];
+  buf ^= 1;
+  return s;
+}
+
 template <typename T>
 __device__ __forceinline__ void block_sum2(T a, T b, T *red, int &buf, T &A, T &B) {
   a = warp_sum(a);
@@ -221,6 +246,33 @@ __device__ __forceinline__ void block_sum2(T a, T b, T *red, int &buf, T &A, T &
     B += r[4 + k];
   }
   buf ^= 1;
+}
+
+// block_sum2 of the first N threads' values, by block_sum_first's rule in FP64
+template <typename T>
+__device__ __forceinline__ void block_sum2_first(T a, T b, int N, T *red, int &buf, T &A, T &B) {
+  if constexpr (std::is_same<T, double>::value) {
+    const int warp = threadIdx.x >> 5, nw = (N + 31) >> 5;
+    double *r = red + buf * 16;
+    if (warp < nw) {
+      a = warp_sum_first(a, N);
+      b = warp_sum_first(b, N);
+      if ((threadIdx.x & 31) == 0) {
+        r[warp] = a;
+        r[4 + warp] = b;
+      }
+    }
+    __syncthreads();
+    A = r[0];
+    B = r[4];
+    for (int k = 1; k < nw; ++k) {
+      A += r[k];
+      B += r[4 + k];
+    }
+    buf ^= 1;
+  } else {
+    block_sum2(a, b, red, buf, A, B);
+  }
 }
 
 template <typename T>
@@ -336,6 +388,14 @@ __device__ __forceinline__ void row_axpy(T *row, const T *x, T c, int N) {
   for (; k < N; ++k) row[k] -= c * x[k];
 }
 
+// a - (c1 b + c2 d): in FP64 two instructions instead of three
+__device__ __forceinline__ float axpy2_of(float a, float b, float d, float c1, float c2) {
+  return a - (c1 * b + c2 * d);
+}
+__device__ __forceinline__ double axpy2_of(double a, double b, double d, double c1, double c2) {
+  return fma(-c2, d, fma(-c1, b, a));
+}
+
 // row[k] -= c1 x[k] + c2 y[k]  (x, y 16-byte aligned)
 template <typename T>
 __device__ __forceinline__ void row_axpy2(T *row, const T *x, const T *y, T c1, T c2, int N) {
@@ -350,9 +410,9 @@ __device__ __forceinline__ void row_axpy2(T *row, const T *x, const T *y, T c1, 
       ld4(y + k + u, d[u], d[u + 1], d[u + 2], d[u + 3]);
     }
 #pragma unroll
-    for (int u = 0; u < CH; ++u) row[k + u] = a[u] - (c1 * b[u] + c2 * d[u]);
+    for (int u = 0; u < CH; ++u) row[k + u] = axpy2_of(a[u], b[u], d[u], c1, c2);
   }
-  for (; k < N; ++k) row[k] -= c1 * x[k] + c2 * y[k];
+  for (; k < N; ++k) row[k] = axpy2_of(row[k], x[k], y[k], c1, c2);
 }
 
 // sum_k row[k] x[k] with four accumulators (x 16-byte aligned)
@@ -424,7 +484,8 @@ __device__ __forceinline__ T hop_pf_ratio(const SysDev &S, const WSmem<T> &sm, i
   }
   if (!S.n_hidden) {
     mlp = (T)0;
-    return block_sum(prod, sm.red, buf);
+    if constexpr (std::is_same<T, double>::value) return block_sum_first(prod, N, sm.red, buf);
+    else return block_sum(prod, sm.red, buf);
   }
   const int sp = (e >= N) ? Ns : 0;
   const T part = mlp_log_ratio_part(S, sm, t + sp, sm.ele[e] + sp, -1, -1, tid, NT);
@@ -495,7 +556,7 @@ __device__ T exchange_pf_ratio(const SysDev &S, const WSmem<T> &sm, int n, int m
     const T part = mlp_log_ratio_part(S, sm, i + Ns, i, j, j + Ns, tid, NT);
     block_sum3(a22, a12, part, sm.red, buf, A22, A12, mlp);
   } else {
-    block_sum2(a22, a12, sm.red, buf, A22, A12);
+    block_sum2_first(a22, a12, N, sm.red, buf, A22, A12);
     mlp = (T)0;
   }
   const T A11 = vB[n];
@@ -521,8 +582,8 @@ __device__ void row_update(const SysDev &S, const WSmem<T> &sm, int n, const T *
   T *vB = sm.vec + VMC_MAX_N;
   if (tid < N) vB[tid] = col_dot(sm.minv, ldm, tid, vA, N);
   __syncthreads();
-  const T inv = (T)1 / vB[n];
   if (tid < N) {
+    const T inv = (T)1 / vB[n];
     T *row = sm.minv + tid * ldm;
     const T c = row[n] * inv;
     row_axpy(row, vB, c, N);
@@ -543,8 +604,8 @@ __device__ void col_update(const SysDev &S, const WSmem<T> &sm, int m, const T *
     vC[tid] = sm.minv[m * ldm + tid];
   }
   __syncthreads();
-  const T inv = (T)1 / vB[m];
   if (tid < N) {
+    const T inv = (T)1 / vB[m];
     T *row = sm.minv + tid * ldm;
     if (tid == m) {
       for (int k = 0; k < N; ++k) row[k] = vC[k] * inv;
@@ -1114,6 +1175,24 @@ __device__ void delayed_hop_update(const SysDev &S, const WSmem<T> &sm, int e, i
   if (np >= S.delay_k) delayed_flush(S, sm, np);
 }
 
+// Metropolis decision u < (r exp(d))^2 in FP64, u = u24 / 2^24.  An FP64
+// exponential is some thirty instructions of 64 cycles on a proposal's serial
+// path, so FP32 decides where it can: for |d| <= 16 the product's square there
+// is within 3e-6 of the exact one (2^-24 of r, (16 + 2) 2^-24 of the
+// exponential, doubled by the square), and only a u within 1e-5 of it takes
+// the FP64 form.  The decision is always FP64's.
+__device__ __forceinline__ bool accept_hop(uint32_t u24, double r, double d) {
+  const float u = (float)u24 * (1.0f / 16777216.0f);   // exact
+  const float df = (float)d, q = (float)r * expf(df);
+  const float q2 = q * q;
+  if (fabsf(df) <= 16.0f && q2 >= 1e-30f && q2 <= 1e30f) {
+    if (u < q2 * (1.0f - 1e-5f)) return true;
+    if (u > q2 * (1.0f + 1e-5f)) return false;
+  }
+  const double ratio = r * exp(d);
+  return (double)u < ratio * ratio;
+}
+
 // ---------------------------------------------------------------------------
 // One Metropolis proposal (Sec. 3.1.2).  Every thread runs it; decisions are
 // uniform across the block.
@@ -1178,11 +1257,14 @@ __device__ void propose(const SysDev &S, const WSmem<T> &sm, uint2 key, uint32_t
   // Kondo local spins hold one electron each: no hop enters or leaves them
   if (S.lsite && (S.lsite[t] | S.lsite[rs])) return;
   mc.hop_t++;
-  // P(x')/P(x): one thread evaluates it; the barrier inside hop_pf_ratio publishes it.
+  // P(x')/P(x), or its logarithm for accept_hop: one thread evaluates it; the
+  // barrier inside hop_pf_ratio publishes it.
   const int slot = buf;
-  if (tid == 0)
-    sm.bc[slot] = corr_factor<T>(corr_hop_v(sm.occ, sm.jf, gtab<T>(S), Ns, s, rs, t,
-                                            vtab<T>(S)[(size_t)rs * Ns + t]));
+  const bool screen = std::is_same<T, double>::value && !S.n_hidden;
+  if (tid == 0) {
+    const T d = corr_hop_v(sm.occ, sm.jf, gtab<T>(S), Ns, s, rs, t, vtab<T>(S)[(size_t)rs * Ns + t]);
+    sm.bc[slot] = screen ? d : corr_factor<T>(d);
+  }
   // rows t and r of v for the Jastrow-field update, fetched while the ratio is formed
   T vt[2], vr[2];
 #pragma unroll
@@ -1193,8 +1275,12 @@ __device__ void propose(const SysDev &S, const WSmem<T> &sm, uint2 key, uint32_t
   }
   T fval, mlp;
   const T rpf = hop_pf_ratio(S, sm, e, t, fval, buf, mlp, np);
-  const T ratio = S.n_hidden ? rpf * sm.bc[slot] * exp_t<T>(mlp) : rpf * sm.bc[slot];
-  if (!(u < ratio * ratio)) return;
+  if (screen) {
+    if (!accept_hop(r.w >> 8, (double)rpf, (double)sm.bc[slot])) return;
+  } else {
+    const T ratio = S.n_hidden ? rpf * sm.bc[slot] * exp_t<T>(mlp) : rpf * sm.bc[slot];
+    if (!(u < ratio * ratio)) return;
+  }
   if (tid < N) sm.vec[tid] = fval;
   __syncthreads();
   bool done = false;
@@ -1666,6 +1752,17 @@ __device__ void measure(const SysDev &S, const WSmem<T> &sm, int w, int row, int
     }
   };
   const int tix = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+  // FP64: the terms whose correlation-factor ratio is still to come, one per lane
+  int slot = 0;
+  T late = (T)0, late_v = (T)0;
+  int2 late_ij = make_int2(-1, 0);   // target site; source site + Ns spin
+  auto late_add = [&]() {
+    if (late_ij.x >= 0) {
+      const int sp = late_ij.y >= Ns, j = late_ij.y - (sp ? Ns : 0);
+      eo += late * corr_factor<T>(corr_hop_v(sm.occ, sm.jf, gtab<T>(S), Ns, sp, j, late_ij.x, late_v));
+    }
+    late_ij.x = -1;
+  };
   if (warp < Ns) fetch(warp, gu, gd, jl, tl, vl);
   for (int i = warp; i < Ns; i += NWARP) {
     const int inext = i + NWARP;
@@ -1702,22 +1799,45 @@ __device__ void measure(const SysDev &S, const WSmem<T> &sm, int w, int row, int
             any |= eur[r] >= 0 || edr[r] >= 0;
           }
           if (!any) continue;
-          // Branch-free: absent terms read column / row 0 and are masked, so
-          // all 32 shared loads can be in flight together (gu, gd are 0 for
-          // q >= N; q is clamped to a valid row).
           T p[8];
+          if constexpr (std::is_same<T, double>::value) {
+            // FP64: the pipe is what counts, so only the terms there are (the
+            // branches are uniform over the warp).  With the factors below
+            // evaluated four groups at a time: 1024 walkers at 8 x 8, four
+            // measurements 1.09 -> 0.55 ms; at 16 x 16 (N = 112) one 1.84 -> 1.37.
 #pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            const int cu = max(eur[r], 0), rd = max(edr[r] - N, 0);
-            T su = (T)0, sd = (T)0;
+            for (int r = 0; r < 4; ++r) {
+              p[2 * r] = p[2 * r + 1] = 0.0;
+              if (eur[r] >= 0) {
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const int q = min(lane + 32 * u, N - 1);
-              su += gu[u] * sm.minv[q * ldm + cu];
-              sd += gd[u] * sm.minv[rd * ldm + q];
+                for (int u = 0; u < 4; ++u)
+                  if (32 * u < N)
+                    p[2 * r] += gu[u] * sm.minv[min(lane + 32 * u, N - 1) * ldm + eur[r]];
+              }
+              if (edr[r] >= 0) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                  if (32 * u < N)
+                    p[2 * r + 1] += gd[u] * sm.minv[(edr[r] - N) * ldm + min(lane + 32 * u, N - 1)];
+              }
             }
-            p[2 * r] = eur[r] >= 0 ? su : (T)0;
-            p[2 * r + 1] = edr[r] >= 0 ? sd : (T)0;
+          } else {
+            // Branch-free: absent terms read column / row 0 and are masked, so
+            // all 32 shared loads can be in flight together (gu, gd are 0 for
+            // q >= N; q is clamped to a valid row).
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+              const int cu = max(eur[r], 0), rd = max(edr[r] - N, 0);
+              T su = (T)0, sd = (T)0;
+#pragma unroll
+              for (int u = 0; u < 4; ++u) {
+                const int q = min(lane + 32 * u, N - 1);
+                su += gu[u] * sm.minv[q * ldm + cu];
+                sd += gd[u] * sm.minv[rd * ldm + q];
+              }
+              p[2 * r] = eur[r] >= 0 ? su : (T)0;
+              p[2 * r + 1] = edr[r] >= 0 ? sd : (T)0;
+            }
           }
           const T sum = reduce8_transposed(p, lane);
           // this lane's term: r = tix >> 1, spin = tix & 1
@@ -1734,6 +1854,23 @@ __device__ void measure(const SysDev &S, const WSmem<T> &sm, int w, int row, int
                   edr[rr] >= 0 ? mlp_log_ratio_part(S, sm, i + Ns, jr[rr] + Ns, -1, -1, lane, 32) : (T)0;
             }
             lm = reduce8_transposed(mq, lane);
+          }
+          if constexpr (std::is_same<T, double>::value) {
+            if (!S.n_hidden) {
+              // every lane of a quad holds its term's sum: lane slot of the
+              // quad keeps it, and four groups' factors are evaluated together
+              if ((lane & 3) == slot && el >= 0) {
+                late = -sel4(tr, r) * sum;
+                late_v = sel4(vr, r);
+                late_ij = make_int2(i, j + (sp ? Ns : 0));
+                mc.meas_hop++;
+              }
+              if (++slot == 4) {
+                late_add();
+                slot = 0;
+              }
+              continue;
+            }
           }
           if ((lane & 3) == 0 && el >= 0) {
             const T c = corr_factor<T>(corr_hop_v(sm.occ, sm.jf, gtab<T>(S), Ns, sp, j, i, sel4(vr, r)));
@@ -1752,6 +1889,7 @@ __device__ void measure(const SysDev &S, const WSmem<T> &sm, int w, int row, int
     tl = ntl;
     vl = nvl;
   }
+  if constexpr (std::is_same<T, double>::value) late_add();
   // --- Heisenberg exchange: J/2 (S+_a S-_b + S-_a S+_b) = -J/2 x (labelled swap ratio).
   // The terms are taken by the site b that receives the up electron (b holds
   // exactly a down electron m, a exactly an up electron n).  The new row of
