@@ -34,6 +34,10 @@ struct SysHost {
 
 }  // namespace
 
+// long long words of vmc_measure's per-walker values: proposals, acceptances,
+// rebuilds, drift (FP64), and eight move counts
+constexpr size_t STAT_WORDS = 12;
+
 struct vmc_ctx {
   int n_sys = 0;
   int precision = 0;
@@ -45,6 +49,7 @@ struct vmc_ctx {
   int2 *d_work = nullptr;
   int n_work = 0;
   int *d_work_ctr = nullptr;
+  int *status_all = nullptr;  // [systems x walkers] VMC_ST_* bits
   size_t smem_sample = 0, smem_init = 0;
   int n_max = 1;              // largest N of the systems
   int init_form = VMC_INIT_BLOCKED;   // how from-scratch inverses are formed
@@ -367,6 +372,18 @@ int periodic_rebuild(vmc_ctx *c) {
 // Every inverse current before it is read: the full rebuild after a parameter
 // or configuration change, else the periodic rebuild the last vmc_sample left
 // pending (a full rebuild makes that one moot).
+// Every walker's status bits, all systems' in one copy: a wait and a copy per
+// system were 8 us each (64 systems: 0.5 ms a call).
+int status_bits(vmc_ctx *c, int *bad) {
+  size_t n = 0;
+  for (auto &s : c->sys) n += s.W;
+  std::vector<int> st(n);
+  CKC(cudaMemcpyAsync(st.data(), c->status_all, sizeof(int) * n, cudaMemcpyDeviceToHost, c->st));
+  CKC(cudaStreamSynchronize(c->st));
+  for (int b : st) *bad |= b;
+  return VMC_OK;
+}
+
 int ensure_init(vmc_ctx *c, bool redraw_illcond = false) {
   bool any = false;
   for (auto &s : c->sys) any |= s.dirty;
@@ -389,13 +406,8 @@ int ensure_init(vmc_ctx *c, bool redraw_illcond = false) {
                           c->init_form, c->n_max, 0, 0, c->smem_init, c->st, &c->n_launch));
   }
   int bad = 0;
-  for (auto &s : c->sys) {
-    std::vector<int> st(s.W);
-    CKC(cudaMemcpyAsync(st.data(), s.dev.status, sizeof(int) * s.W, cudaMemcpyDeviceToHost, c->st));
-    CKC(cudaStreamSynchronize(c->st));
-    for (int w = 0; w < s.W; ++w) bad |= st[w];
-    s.dirty = false;
-  }
+  CK(status_bits(c, &bad));
+  for (auto &s : c->sys) s.dirty = false;
   if ((bad & VMC_ST_SINGULAR) || (redraw_illcond && (bad & VMC_ST_ILLCOND))) {
     for (auto &s : c->sys) s.dirty = true;
     return VMC_ESINGULAR;
@@ -566,6 +578,10 @@ int create_impl(vmc_ctx **out, int n_sys, const vmc_model *models, const int32_t
     delete c;
     return e;
   };
+  // status words of every system's walkers, side by side
+  if (o->n_walkers > 0 &&
+      (rc = dupload(c, &c->status_all, (const int *)nullptr, (size_t)n_sys * o->n_walkers)))
+    return fail(rc);
   for (int si = 0; si < n_sys; ++si) {
     const vmc_model &m = models[si];
     const vmc_layout &l = layouts[si];
@@ -739,15 +755,17 @@ int create_impl(vmc_ctx **out, int n_sys, const vmc_model *models, const int32_t
     if ((rc = dupload(c, &d.ctr, (const unsigned long long *)nullptr, W))) return fail(rc);
     if ((rc = dupload(c, &d.logdet, (const double *)nullptr, W))) return fail(rc);
     if ((rc = dupload(c, &d.detsign, (const int *)nullptr, W))) return fail(rc);
-    if ((rc = dupload(c, &d.n_prop, (const long long *)nullptr, W))) return fail(rc);
-    if ((rc = dupload(c, &d.n_acc, (const long long *)nullptr, W))) return fail(rc);
-    if ((rc = dupload(c, &d.cnt, (const long long *)nullptr, 8 * W))) return fail(rc);
-    if ((rc = dupload(c, &d.n_rec, (const long long *)nullptr, W))) return fail(rc);
     if ((rc = dupload(c, &d.acc_since, (const int *)nullptr, W))) return fail(rc);
-    if ((rc = dupload(c, &d.status, (const int *)nullptr, W))) return fail(rc);
-    if ((rc = dupload(c, &d.drift, (const double *)nullptr, W))) return fail(rc);
+    d.status = c->status_all + (size_t)si * W;
+    // the counters and E of a system side by side: vmc_measure reads them in one copy
     const size_t rows_cap = W * s.max_samples;
-    if ((rc = dupload(c, &d.E, (const double *)nullptr, rows_cap))) return fail(rc);
+    if ((rc = dupload(c, &d.n_prop, (const long long *)nullptr, STAT_WORDS * W + rows_cap)))
+      return fail(rc);
+    d.n_acc = d.n_prop + W;
+    d.n_rec = d.n_prop + 2 * W;
+    d.drift = (double *)(d.n_prop + 3 * W);
+    d.cnt = d.n_prop + 4 * W;
+    d.E = (double *)(d.n_prop + STAT_WORDS * W);
     if ((rc = dalloc(c, &d.O, (size_t)esize * rows_cap * s.ldO))) return fail(rc);
     int acc_len = 0;
     smem64 = std::max(smem64, vmc_walker_smem(0, s.N, s.Ns, s.Np, H, 0, &acc_len, 0));
@@ -926,12 +944,7 @@ int vmc_sample(vmc_ctx *c, int32_t n_warmup, int32_t n_samples, int32_t sweeps_b
     if (launches > 0) c->rebuild_pending = true;
   }
   int bad = 0;
-  for (auto &s : c->sys) {
-    std::vector<int> st(s.W);
-    CKC(cudaMemcpyAsync(st.data(), s.dev.status, sizeof(int) * s.W, cudaMemcpyDeviceToHost, c->st));
-    CKC(cudaStreamSynchronize(c->st));
-    for (int w = 0; w < s.W; ++w) bad |= st[w];
-  }
+  CK(status_bits(c, &bad));
   if (bad & VMC_ST_TIMEOUT) return VMC_ETIMEOUT;
   if (bad & VMC_ST_SINGULAR) return VMC_ESINGULAR;
   if (bad & VMC_ST_NUMERIC) return VMC_ENUMERIC;
@@ -942,20 +955,17 @@ int vmc_measure(vmc_ctx *c, int32_t system, vmc_stats *out) {
   if (!sys_ok(c, system) || !out) return VMC_EINVAL;
   SysHost &s = c->sys[system];
   memset(out, 0, sizeof(*out));
-  std::vector<long long> np(s.W), na(s.W);
-  std::vector<int> st(s.W);
-  std::vector<double> dr(s.W);
-  CKC(cudaMemcpyAsync(np.data(), s.dev.n_prop, sizeof(long long) * s.W, cudaMemcpyDeviceToHost, c->st));
-  CKC(cudaMemcpyAsync(na.data(), s.dev.n_acc, sizeof(long long) * s.W, cudaMemcpyDeviceToHost, c->st));
-  CKC(cudaMemcpyAsync(st.data(), s.dev.status, sizeof(int) * s.W, cudaMemcpyDeviceToHost, c->st));
-  CKC(cudaMemcpyAsync(dr.data(), s.dev.drift, sizeof(double) * s.W, cudaMemcpyDeviceToHost, c->st));
-  std::vector<long long> cn(8 * (size_t)s.W), nr(s.W);
-  CKC(cudaMemcpyAsync(cn.data(), s.dev.cnt, sizeof(long long) * cn.size(), cudaMemcpyDeviceToHost, c->st));
-  CKC(cudaMemcpyAsync(nr.data(), s.dev.n_rec, sizeof(long long) * s.W, cudaMemcpyDeviceToHost, c->st));
-  std::vector<double> E(s.rows);
-  if (s.rows)
-    CKC(cudaMemcpyAsync(E.data(), s.dev.E, sizeof(double) * s.rows, cudaMemcpyDeviceToHost, c->st));
+  const size_t W = s.W;
+  std::vector<long long> words(STAT_WORDS * W + s.rows);
+  std::vector<int> st(W);
+  CKC(cudaMemcpyAsync(words.data(), s.dev.n_prop, sizeof(long long) * words.size(),
+                      cudaMemcpyDeviceToHost, c->st));
+  CKC(cudaMemcpyAsync(st.data(), s.dev.status, sizeof(int) * W, cudaMemcpyDeviceToHost, c->st));
   CKC(cudaStreamSynchronize(c->st));
+  const long long *np = words.data(), *na = np + W, *nr = np + 2 * W, *cn = np + 4 * W;
+  std::vector<double> dr(W), E(s.rows);
+  memcpy(dr.data(), np + 3 * W, sizeof(double) * W);
+  if (s.rows) memcpy(E.data(), np + STAT_WORDS * W, sizeof(double) * s.rows);
   for (int w = 0; w < s.W; ++w) {
     out->n_proposals += np[w];
     out->n_accepted += na[w];
