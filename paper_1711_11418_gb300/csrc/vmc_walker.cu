@@ -2626,7 +2626,10 @@ cudaError_t vmc_launch_init(const SysDev *d_sys, const int2 *d_work, int n_work,
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const int nth = form == VMC_INIT_BLOCKED ? vmc_gj::gj_threads(n_max)
+  // by panels: up to four walkers per SM take at least NT threads, for the work
+  // per site around the elimination (N = 38 has 96 threads of its own)
+  const int panel_nth = vmc_gj::gj_threads(n_max);
+  const int nth = form == VMC_INIT_BLOCKED ? (n_work <= 4 * nsm && panel_nth < NT ? NT : panel_nth)
                   : form == VMC_INIT_DF    ? NT
                                            : vmc_gj::gj_step_threads(n_max);
   const InitKernel kern = init_kernel(precision, form, nth);
