@@ -319,13 +319,14 @@ int upload_sysdesc(vmc_ctx *c) {
 }
 
 // Delay depth k: shared-memory size and grid of the sweep kernel follow it.
-int set_delay_impl(vmc_ctx *c, int k) {
+// k: pending updates; spec_b: proposals formed together.  Sets the sweep's launch shape.
+int set_sweep_impl(vmc_ctx *c, int k, int spec_b) {
   if (k < 0 || k > VMC_DELAY_MAX) return VMC_EINVAL;
   const int kd = k <= 1 ? 0 : k;
   size_t smem = 0;
   for (auto &s : c->sys)
-    smem = std::max(smem, vmc_walker_smem(c->precision == VMC_FP64 ? 0 : 1, s.N, s.Ns, s.Np,
-                                          s.dev.n_hidden, kd, nullptr,
+    smem = std::max(smem, vmc_walker_smem(c->precision == VMC_FP64 ? 0 : 1, s.N, s.Ns,
+                                          s.dev.acc_len, s.dev.n_hidden, kd, spec_b,
                                           c->precision == VMC_MIXED));
   if (smem > c->smem_cap) return VMC_EINVAL;
   int dev = 0, nsm = 0;
@@ -342,7 +343,11 @@ int set_delay_impl(vmc_ctx *c, int k) {
         const size_t mb = ((size_t)s.N * s.ldm * 4 + 127) / 128 * 128;
         CKC(cudaMemsetAsync(s.dev.minv_lo, 0, (size_t)s.W * mb, c->st));
       }
-  for (auto &s : c->sys) s.dev.delay_k = kd;
+  for (auto &s : c->sys) {
+    s.dev.delay_k = kd;
+    s.dev.spec_b = spec_b;
+  }
+  c->spec_b = spec_b;
   c->smem_sample = smem;
   c->grid_sample = std::min(c->n_work, nsm * occ);
   c->delay_k = k;
@@ -571,7 +576,7 @@ int create_impl(vmc_ctx **out, int n_sys, const vmc_model *models, const int32_t
   c->sys.resize(n_sys);
   const int esize = o->precision == VMC_FP64 ? 8 : 4;
   int rc = VMC_OK;
-  size_t smem64 = 0, smem32 = 0;
+  size_t smem64 = 0, smem64g = 0, smem64w = 0, smem32 = 0;
   bool exchange = false;      // some system has exchange terms
   auto fail = [&](int e) {
     ctx_free(c);
@@ -767,10 +772,11 @@ int create_impl(vmc_ctx **out, int n_sys, const vmc_model *models, const int32_t
     d.cnt = d.n_prop + 4 * W;
     d.E = (double *)(d.n_prop + STAT_WORDS * W);
     if ((rc = dalloc(c, &d.O, (size_t)esize * rows_cap * s.ldO))) return fail(rc);
-    int acc_len = 0;
-    smem64 = std::max(smem64, vmc_walker_smem(0, s.N, s.Ns, s.Np, H, 0, &acc_len, 0));
-    smem32 = std::max(smem32, vmc_walker_smem(1, s.N, s.Ns, s.Np, H, 0, &acc_len, 1));
-    d.acc_len = acc_len;
+    d.acc_len = vmc_walker_acc_len(s.Np);
+    smem64 = std::max(smem64, vmc_walker_smem(0, s.N, s.Ns, d.acc_len, H, 0, 1, 0));
+    smem64g = std::max(smem64g, vmc_walker_smem(0, s.N, s.Ns, 0, H, 0, 1, 0));
+    smem64w = std::max(smem64w, vmc_walker_smem(0, s.N, s.Ns, d.acc_len, H, 0, 2, 0));
+    smem32 = std::max(smem32, vmc_walker_smem(1, s.N, s.Ns, d.acc_len, H, 0, 1, 1));
     exchange |= m.n_J > 0;
     if (vmc_launch_expand(&d, c->st, &c->n_launch) != cudaSuccess) return fail(VMC_ECUDA);
     // seeded random placement
@@ -794,7 +800,9 @@ int create_impl(vmc_ctx **out, int n_sys, const vmc_model *models, const int32_t
     int optin = 0;
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     c->smem_cap = optin > 4096 ? (size_t)optin - 4096 : 0;
-    if (c->smem_sample > c->smem_cap || c->smem_init > (size_t)optin) return fail(VMC_EINVAL);
+    // (batches of proposals have to fit as well)
+    if ((c->precision == VMC_FP64 ? smem64w : smem32) > c->smem_cap || c->smem_init > (size_t)optin)
+      return fail(VMC_EINVAL);
     if (vmc_walker_set_smem_limits(c->smem_cap, c->smem_cap, c->smem_init) != cudaSuccess) {
       cudaGetLastError();
       return fail(VMC_EINVAL);  // does not fit in shared memory
@@ -815,9 +823,13 @@ int create_impl(vmc_ctx **out, int n_sys, const vmc_model *models, const int32_t
   if ((rc = dalloc(c, &c->d_scalar, sizeof(double) * 8))) return fail(rc);
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const int occ = std::max(1, vmc_sample_occupancy(c->precision, c->smem_sample));
-  c->grid_sample = std::min(c->n_work, nsm * occ);
-  if ((rc = set_delay_impl(c, o->delay_k))) return fail(rc);
+  // Plain form: the O rows are accumulated in their global rows where that lets
+  // a second CTA onto the SM (FP64 M^-1 of N = 112 with 1069 parameters: 117
+  // against 110 KB a walker; 1024 walkers, a sweep and a measurement 8.4 -> 6.1 ms).
+  if (c->precision == VMC_FP64 && vmc_sample_occupancy(0, smem64) < 2 &&
+      vmc_sample_occupancy(0, smem64g) >= 2)
+    for (SysHost &s : c->sys) s.dev.acc_len = 0;
+  if ((rc = set_sweep_impl(c, o->delay_k, c->spec_b))) return fail(rc);
   c->recompute_every = o->recompute_every > 0 ? o->recompute_every
                        : (o->recompute_every == 0 && o->precision == VMC_MIXED) ? 64 : 0;
   // Initial inverses; re-draw placements whose M is singular (bounded).
@@ -1533,7 +1545,7 @@ int vmc_lanczos_alpha(const double *h, double *alpha, double *E1) {
 
 int vmc_set_delay(vmc_ctx *c, int32_t k) {
   if (!c || (projected(c) && k > 1)) return VMC_EINVAL;
-  return set_delay_impl(c, k);
+  return set_sweep_impl(c, k, c->spec_b);
 }
 
 int vmc_set_projection(vmc_ctx *c, int32_t n_ops, const int32_t *perm, const int8_t *sign,
@@ -1626,7 +1638,7 @@ int vmc_tune_delay(vmc_ctx *c, int32_t sweeps, const int32_t *cand, int32_t n_ca
   int rc = VMC_OK;
   for (int q = 0; q < n_cand && rc == VMC_OK; ++q) {
     if (ms) ms[q] = -1.0;
-    if (set_delay_impl(c, cand[q]) != VMC_OK) continue;
+    if (set_sweep_impl(c, cand[q], c->spec_b) != VMC_OK) continue;
     cudaEventRecord(e0, c->st);
     rc = vmc_sample(c, 0, 1, sweeps);
     cudaEventRecord(e1, c->st);
@@ -1648,18 +1660,16 @@ int vmc_tune_delay(vmc_ctx *c, int32_t sweeps, const int32_t *cand, int32_t n_ca
   cudaEventDestroy(e1);
   c->recompute_every = rec;
   if (rc != VMC_OK || best < 0) {
-    set_delay_impl(c, prev);
+    set_sweep_impl(c, prev, c->spec_b);
     return rc != VMC_OK ? rc : VMC_EINVAL;
   }
   *chosen = best;
-  return set_delay_impl(c, best);
+  return set_sweep_impl(c, best, c->spec_b);
 }
 
 int vmc_set_proposal_batch(vmc_ctx *c, int32_t b) {
   if (!c || b < 1 || b > VMC_SPEC_MAX) return VMC_EINVAL;
-  for (auto &s : c->sys) s.dev.spec_b = b;
-  c->spec_b = b;
-  return VMC_OK;
+  return set_sweep_impl(c, c->delay_k, b);
 }
 
 int32_t vmc_get_proposal_batch(vmc_ctx *c) { return c ? c->spec_b : -1; }

@@ -156,8 +156,10 @@ cudaError_t vmc_launch_corr_reduce(const double *part, int n_part, const int *cn
                                    long long *n_launch);
 // with_lo: the mixed form's sweep keeps the low words of its double-float
 // M^-1 in shared memory as well.
-size_t vmc_walker_smem(int precision, int N, int Ns, int Np, int H, int kd, int *acc_len,
+// acc_len: words of the O row accumulated in shared memory (0: in its global row).
+size_t vmc_walker_smem(int precision, int N, int Ns, int acc_len, int H, int kd, int spec_b,
                        int with_lo);
+int vmc_walker_acc_len(int Np);
 size_t vmc_init_smem(int N, int Ns, int form);
 int vmc_sample_occupancy(int precision, size_t smem);
 // the mixed form's 168-register sweep variant (vmc_sweep3.cu)

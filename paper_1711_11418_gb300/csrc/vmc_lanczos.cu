@@ -43,7 +43,7 @@
 // What bounds it: (3) issue, about 40 instructions per pair and 2.5e5 pairs a
 // walker at 16 x 16; (1) the loads that feed its multiply-adds.  Every pair
 // reading four tables of the slot, and tables formed entry by entry from
-// strided loads, took 35.9 ms for 1024 walkers of 16 x 16 (FP32); 4.7 ms so.
+// strided loads, took 35.9 ms for 1024 walkers of 16 x 16 (FP32); 4.9 ms so.
 #include "vmc_common.cuh"
 #include "vmc_dev.cuh"
 

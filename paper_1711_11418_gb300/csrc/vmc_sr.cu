@@ -285,7 +285,7 @@ __global__ void k_mirror_shift(double *S, int Np, double shift_rel, double shift
 // right-hand side.  What bounds it: the chain of n pivots (about 1000 clocks
 // each: a reciprocal, a column, a barrier, eight multiply-adds on a pipe that
 // takes 64 clocks for a warp's) and the FP64 pipe for n^3 / 3 multiply-adds.
-// n = 1069: panels 2.37 -> 0.8 ms, both triangular solves 1.32 -> 0.15 ms.
+// n = 1069: panels 2.37 -> 1.04 ms, both triangular solves 1.32 -> 0.16 ms.
 constexpr int CB = 32;
 constexpr int PT = 128;    // threads of k_chol_panel
 

@@ -90,7 +90,8 @@ __device__ __forceinline__ void block_invert(float (*D)[GB + 1], float (*rowk)[G
 //   i in K:      A_ij <- B
 //   i not in K:  A_ij <- (j in K ? 0 : A_ij) - sum_l C_il B_lj.
 // What bounds it: latency (a 32-step inversion, two small products, one tile);
-// n = 1069: 39 us in two launches per step -> 9.5 us.
+// n = 1069: 39 us in two launches per step -> 16 us from cold caches; the whole SR
+// step of that size 2.17 -> 1.26 ms.
 __global__ void __launch_bounds__(256) k_gj_step(float *A, int n, int k0, int nb, const float *R,
                                                  const float *C, float *Rn, float *Cn) {
   __shared__ float D[GB][GB + 1];

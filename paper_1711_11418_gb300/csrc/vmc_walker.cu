@@ -117,7 +117,7 @@ __device__ __forceinline__ void fence_proxy_async() {
 template <typename T>
 struct WSmem {
   T *minv;      // N x ldm
-  T *vec;       // 8 x VMC_MAX_N: block vectors vA..vD, or 2 per warp
+  T *vec;       // 8 (or 4) x VMC_MAX_N: block vectors vA..vD and more, or one per warp
   T *acc;       // O-row accumulator (acc_len); shares its space with ut/vt
   T *ut;        // delayed updates: u_i = ut[i*N ..], i < pending (measurement flushes first)
   T *vt;        //                  v_i = vt[i*N ..]
@@ -139,13 +139,20 @@ struct WSmem {
 constexpr int RB = 32;
 
 template <typename T>
+__host__ __device__ constexpr bool layout_wide(int delay_k, int spec_b) {
+  return sizeof(T) == 4 || delay_k > 1 || spec_b > 1;
+}
+
+// wide: eight block vectors, which batches of proposals, delayed updates and
+// the mixed form use; the plain form's proposals one at a time use four.
+template <typename T>
 __host__ __device__ size_t walker_layout(int N, int Ns, int acc_len, int H, int kd, bool lo,
-                                         unsigned char *base, WSmem<T> *sm) {
+                                         bool wide, unsigned char *base, WSmem<T> *sm) {
   const int ldm = (N % 2) ? N : N + 1;
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 16); return o; };
   const size_t o_minv = take(minv_bytes(N, ldm, sizeof(T)));
-  const size_t o_vec = take(sizeof(T) * 8 * VMC_MAX_N);
+  const size_t o_vec = take(sizeof(T) * (wide ? 8 : 4) * VMC_MAX_N);
   const size_t dly = (kd > 1) ? sizeof(T) * 2 * (size_t)kd * N : 0;
   // the O-row accumulator; also the delayed pairs, or a proposal batch's
   // per-warp partial sums (NWARP x 32 values), none of which live together
@@ -1897,7 +1904,7 @@ __device__ void measure(const SysDev &S, const WSmem<T> &sm, int w, int row, int
   // w = R^T M^-1 = g_b + (f(b, a) - f(b, b)) M^-1[m,:] with g_b = f(b, r_dn)^T M^-1
   // formed once per site by one warp (lanes over columns), and each term is
   // the 2 x 2 determinant of exchange_pf_ratio in O(N).
-  T *R = sm.vec + (2 * warp) * VMC_MAX_N;
+  T *R = sm.vec + warp * VMC_MAX_N;
   __syncthreads();   // vec area switches from proposal use to per-warp use
   if (S.n_J > 0) {
     const unsigned full = 0xffffffffu;
@@ -2098,7 +2105,8 @@ __global__ void __launch_bounds__(NT, MINB) k_sample(const SysDev *systems, cons
     const int w = wk.y;
     const int N = S.N, Ns = S.Ns, Ne = S.Ne, ldm = S.ldm, tid = threadIdx.x;
     WSmem<T> sm;
-    walker_layout<T>(N, Ns, S.acc_len, S.n_hidden, S.delay_k, S.minv_lo != nullptr, smem_raw, &sm);
+    walker_layout<T>(N, Ns, S.acc_len, S.n_hidden, S.delay_k, S.minv_lo != nullptr,
+                     layout_wide<T>(S.delay_k, S.spec_b), smem_raw, &sm);
     // --- load the walker: M^-1 block by a TMA bulk copy, configuration and
     // Jastrow field by plain loads while the copy is in flight
     const uint32_t nbytes = (uint32_t)minv_bytes(N, ldm, sizeof(T));
@@ -2490,7 +2498,8 @@ __global__ void __launch_bounds__(NT) k_eval_ratios(const SysDev *systems, int s
   load_sys(&S, systems + sys);
   const int N = S.N, Ns = S.Ns, Ne = S.Ne, ldm = S.ldm, tid = threadIdx.x;
   WSmem<T> sm;
-  walker_layout<T>(N, Ns, S.acc_len, S.n_hidden, 0, false, smem_raw, &sm);
+  walker_layout<T>(N, Ns, S.acc_len, S.n_hidden, 0, false, layout_wide<T>(S.delay_k, S.spec_b),
+                   smem_raw, &sm);
   const size_t nb = minv_bytes(N, ldm, sizeof(T));
   const T *src = (const T *)((const unsigned char *)S.minv + (size_t)w * nb);
   for (int k = tid; k < N * ldm; k += NT) sm.minv[k] = src[k];
@@ -2539,12 +2548,14 @@ __global__ void __launch_bounds__(NT) k_eval_ratios(const SysDev *systems, int s
 // ---------------------------------------------------------------------------
 // Host-side launch wrappers
 // ---------------------------------------------------------------------------
-size_t vmc_walker_smem(int precision, int N, int Ns, int Np, int H, int kd, int *acc_len,
+int vmc_walker_acc_len(int Np) { return (Np <= VMC_ACC_MAX) ? Np : 0; }
+
+size_t vmc_walker_smem(int precision, int N, int Ns, int acc_len, int H, int kd, int spec_b,
                        int with_lo) {
-  const int al = (Np <= VMC_ACC_MAX) ? Np : 0;
-  if (acc_len) *acc_len = al;
-  return precision == 0 ? walker_layout<double>(N, Ns, al, H, kd, false, nullptr, nullptr)
-                        : walker_layout<float>(N, Ns, al, H, kd, with_lo != 0, nullptr, nullptr);
+  return precision == 0
+             ? walker_layout<double>(N, Ns, acc_len, H, kd, false, layout_wide<double>(kd, spec_b),
+                                     nullptr, nullptr)
+             : walker_layout<float>(N, Ns, acc_len, H, kd, with_lo != 0, true, nullptr, nullptr);
 }
 
 int vmc_init_form(int precision, int df, int exchange, int n_max) {

@@ -38,3 +38,21 @@ def test_chain_equals_the_batched_one(Ns, N, scale):
     np.testing.assert_array_equal(ele1, ele4)
     np.testing.assert_array_equal(ctr1, ctr4)
     np.testing.assert_allclose(E1, E4, rtol=1e-9, atol=1e-9 * max(1.0, np.abs(E4).max()))
+
+
+def test_two_walkers_per_sm_equal_the_wide_layout():
+    """16 x 16, N = 112: proposals one at a time take a walker of half an SM's
+    shared memory, with the O rows accumulated in global memory; batches a
+    larger one.  Same chain, E and O."""
+    p = I.square16_hubbard()
+    out = []
+    for batch in (1, 4):
+        with vmc.Context(p, 4, seed=5, max_samples=2) as ctx:
+            ctx.set_proposal_batch(batch)
+            ctx.sample(0, 2, 1)
+            out.append((*ctx.get_samples(), *ctx.get_configs()))
+    (E1, O1, ele1, ctr1), (E4, O4, ele4, ctr4) = out
+    np.testing.assert_array_equal(ele1, ele4)
+    np.testing.assert_array_equal(ctr1, ctr4)
+    np.testing.assert_allclose(E1, E4, rtol=1e-9, atol=1e-9 * np.abs(E4).max())
+    np.testing.assert_allclose(O1, O4, rtol=1e-9, atol=1e-9 * np.abs(O4).max())
