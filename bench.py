@@ -43,12 +43,13 @@ FP64_PEAK_TFLOPS = SMS * FP64_UNITS * 2 * SM_MAX_MHZ * 1e6 / 1e12
 # DRAM bytes (read + write) per launch from one ncu capture (one-pass
 # metrics) of the current kernels at 4096 walkers
 # (profiles/dram_k_sample_k_init_hubbard16x16_w4096.md): a sweep-only launch
-# of k_sample<float> and the full rebuild launch of k_init<float>.
+# of k_sample<float>; and the full rebuild launch of k_init<float>
+# (profiles/time_dram_hubbard16x16.md).
 TRAFFIC_SWEEP_ONLY_4096 = 434.15e6 + 368.07e6
-TRAFFIC_INIT_4096 = 5.54e6 + 366.87e6
+TRAFFIC_INIT_4096 = 6.1e6 + 362.9e6
 # k_corr<float> (pair correlations), DRAM read + write per launch at 4096
-# walkers (profiles/k_corr_float_hubbard16x16_w4096.md).
-TRAFFIC_CORR_4096 = 230.7e6
+# walkers (profiles/time_dram_hubbard16x16.md).
+TRAFFIC_CORR_4096 = 226.4e6 + 0.1e6
 
 
 def hbm_peak_gbs():
@@ -779,7 +780,13 @@ def run_ours(args):
             runs = [ctx.measure_corr(timing=True)[1] for _ in range(5)]
             k_ms = statistics.median(r[0] for r in runs)
             all_ms = statistics.median(r[1] for r in runs)
-            corr = {"k_ms": k_ms, "all_ms": all_ms}
+            # singly occupied sites of each walker (as many of either spin)
+            ele = ctx.get_configs()[0]
+            occ = np.zeros((2, len(ele), prob.Ns), bool)
+            for s in range(2):
+                np.put_along_axis(occ[s], ele[:, s * N:(s + 1) * N].astype(np.int64), True, 1)
+            single = (occ[1] & ~occ[0]).sum(1).astype(np.float64)
+            corr = {"k_ms": k_ms, "all_ms": all_ms, "single2": float((single ** 2).sum())}
         ctx.close()
         others = None if args.no_others else other_workloads(vmc, torch, stream)
 
@@ -849,14 +856,17 @@ def run_ours(args):
                  "kernel": "k_init<float> (FP64 from-scratch inverses)",
                  "ms_in_timed_region": init_ms,
                  "peak_source": "derived: 152 SMs x 2 FP64 FMA units x 2 x 2070 MHz "
-                                "(a DFMA throughput loop measured 1.198 TFLOP/s)"}
+                                "(a DFMA throughput loop measured 1.198 TFLOP/s); the rank-16 "
+                                "updates run in exact 8-bit digits on the tensor cores, so the "
+                                "rate of 2 N^3 per inverse can exceed it"}
     roof, roof2 = (roof_init, roof_sweep) if init_ms > sweep_ms else (roof_sweep, roof_init)
     roof["measured_gemm_tflops"] = peaks
     pair_corr = None
     if corr is not None:
-        # k_corr<float>: per configuration G_up (Ns N^2 FMA) and, for each of
-        # the N sites holding a down electron, G_dn and T (2 N Ns FMA each)
-        fl = 2.0 * 3 * prob.Ns * N * N * args.walkers
+        # k_corr<float>: per configuration G_up and G_dn at the Ns - N sites
+        # without an electron of that spin ((Ns - N) N^2 FMA each) and T between
+        # the singly occupied sites (N FMA per pair)
+        fl = 2.0 * (2 * (prob.Ns - N) * N * N * args.walkers + N * corr["single2"])
         ach_c = fl / (corr["k_ms"] * 1e-3) / 1e12
         pair_corr = {
             "what": "all 6 x Ns^2 pair correlations (c+c up/dn, n n, SzSz, S+S-, S.S) of the "
