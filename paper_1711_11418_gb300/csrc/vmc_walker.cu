@@ -2637,6 +2637,10 @@ cudaError_t vmc_launch_init(const SysDev *d_sys, const int2 *d_work, int n_work,
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  // a walker per SM or fewer: one walker's time is the launch's, and up to N = 48
+  // it is shorter step by step (125 walkers at N = 36, four samples with rebuilds
+  // 1218 -> 1159 us; the gradient of 110 at N = 38 316 -> 308)
+  if (form == VMC_INIT_BLOCKED && n_work <= nsm && n_max <= 48) form = VMC_INIT_STEPS;
   // by panels: up to four walkers per SM take at least NT threads, for the work
   // per site around the elimination (N = 38 has 96 threads of its own)
   const int panel_nth = vmc_gj::gj_threads(n_max);

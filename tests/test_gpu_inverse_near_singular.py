@@ -58,3 +58,20 @@ def test_exactly_singular_is_refused():
             ctx.set_configs(np.array([placement(rng, p.Ns, 32, [0, 1])], np.int32))
             ctx.get_inverse(0)
         assert e.value.code == -4
+
+
+@pytest.mark.parametrize("N", [25, 32, 33, 48])
+@pytest.mark.parametrize("precision", [vmc.FP64, vmc.MIXED])
+def test_small_inverses_by_panels(N, precision):
+    """More walkers than SMs: N <= 48 goes by panels (fewer go step by step)."""
+    p, f, rng = problem(N, 1e-3)
+    W = 320
+    cfg = np.array([placement(rng, p.Ns, N, []) for _ in range(W)], np.int32)
+    with vmc.Context(p, W, seed=5, precision=precision) as ctx:
+        ctx.set_configs(cfg)
+        got = [ctx.get_inverse(w)[0] for w in range(0, W, 40)]
+    for w, X in zip(range(0, W, 40), got):
+        M = f[np.ix_(cfg[w, :N], cfg[w, N:])]
+        ref = np.linalg.inv(M)
+        tol = 64 * N * 2.3e-16 * np.linalg.cond(M) + (2.0 ** -46 if precision == vmc.MIXED else 0.0)
+        assert np.linalg.norm(X - ref) <= tol * np.linalg.norm(ref)
