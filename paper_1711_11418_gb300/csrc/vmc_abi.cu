@@ -50,9 +50,9 @@ struct vmc_ctx {
   int n_work = 0;
   int *d_work_ctr = nullptr;
   int *status_all = nullptr;  // [systems x walkers] VMC_ST_* bits
-  size_t smem_sample = 0, smem_init = 0;
+  size_t smem_sample = 0;
+  InitPlan init;              // how from-scratch inverses are formed and launched
   int n_max = 1;              // largest N of the systems
-  int init_form = VMC_INIT_BLOCKED;   // how from-scratch inverses are formed
   int grid_sample = 0;
   long long n_launch = 0;
   double *d_scalar = nullptr;
@@ -367,9 +367,8 @@ int periodic_rebuild(vmc_ctx *c) {
     CKC(vmc_launch_proj_build(c->d_sys, c->d_work, c->n_work, c->sys[0].dev.n_ops, c->precision,
                               c->n_max, 1, c->recompute_every, c->smem_build, c->st, &c->n_launch));
   else
-    CKC(vmc_launch_init(c->d_sys, c->d_work, c->n_work, c->d_work_ctr + 1, c->precision,
-                        c->init_form, c->n_max, 1, c->recompute_every, c->smem_init, c->st,
-                        &c->n_launch));
+    CKC(vmc_launch_init(c->d_sys, c->d_work, c->n_work, c->d_work_ctr + 1, c->precision, c->init, 1,
+                        c->recompute_every, c->st, &c->n_launch));
   c->rebuild_pending = false;
   return VMC_OK;
 }
@@ -407,8 +406,8 @@ int ensure_init(vmc_ctx *c, bool redraw_illcond = false) {
       CKC(vmc_launch_proj_build(c->d_sys, c->d_work, c->n_work, c->sys[0].dev.n_ops, c->precision,
                                 c->n_max, 0, 0, c->smem_build, c->st, &c->n_launch));
     else
-      CKC(vmc_launch_init(c->d_sys, c->d_work, c->n_work, c->d_work_ctr + 1, c->precision,
-                          c->init_form, c->n_max, 0, 0, c->smem_init, c->st, &c->n_launch));
+      CKC(vmc_launch_init(c->d_sys, c->d_work, c->n_work, c->d_work_ctr + 1, c->precision, c->init,
+                          0, 0, c->st, &c->n_launch));
   }
   int bad = 0;
   CK(status_bits(c, &bad));
@@ -790,10 +789,18 @@ int create_impl(vmc_ctx **out, int n_sys, const vmc_model *models, const int32_t
       return fail(VMC_ECUDA);
   }
   c->smem_sample = (c->precision == VMC_FP64) ? smem64 : smem32;
-  c->init_form = vmc_init_form(c->precision == VMC_FP64 ? 0 : 1,
-                               o->rebuild == VMC_REBUILD_DOUBLE_FLOAT, exchange, c->n_max);
-  for (const SysHost &s : c->sys)
-    c->smem_init = std::max(c->smem_init, vmc_init_smem(s.N, s.Ns, c->init_form));
+  int nsm = 0;
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  c->n_work = n_sys * o->n_walkers;
+  {
+    std::vector<int> N, Ns;
+    for (const SysHost &s : c->sys) {
+      N.push_back(s.N);
+      Ns.push_back(s.Ns);
+    }
+    vmc_init_plan(c->precision == VMC_FP64 ? 0 : 1, o->rebuild == VMC_REBUILD_DOUBLE_FLOAT, exchange,
+                  n_sys, N.data(), Ns.data(), c->n_work, nsm, &c->init);
+  }
   {
     // The sweep kernels may use up to the device's opt-in limit (less the
     // static part): delayed updates enlarge the walker's shared state.
@@ -801,9 +808,9 @@ int create_impl(vmc_ctx **out, int n_sys, const vmc_model *models, const int32_t
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     c->smem_cap = optin > 4096 ? (size_t)optin - 4096 : 0;
     // (batches of proposals have to fit as well)
-    if ((c->precision == VMC_FP64 ? smem64w : smem32) > c->smem_cap || c->smem_init > (size_t)optin)
+    if ((c->precision == VMC_FP64 ? smem64w : smem32) > c->smem_cap || c->init.smem > (size_t)optin)
       return fail(VMC_EINVAL);
-    if (vmc_walker_set_smem_limits(c->smem_cap, c->smem_cap, c->smem_init) != cudaSuccess) {
+    if (vmc_walker_set_smem_limits(c->smem_cap, c->smem_cap, c->init.smem) != cudaSuccess) {
       cudaGetLastError();
       return fail(VMC_EINVAL);  // does not fit in shared memory
     }
@@ -816,13 +823,10 @@ int create_impl(vmc_ctx **out, int n_sys, const vmc_model *models, const int32_t
                    [&](int a, int b) { return c->sys[a].N > c->sys[b].N; });
   for (int s : order)
     for (int w = 0; w < c->sys[s].W; ++w) work.push_back(make_int2(s, w));
-  c->n_work = (int)work.size();
   if ((rc = dupload(c, &c->d_work, work.data(), work.size()))) return fail(rc);
   if ((rc = dalloc(c, &c->d_work_ctr, sizeof(int) * 4))) return fail(rc);
   if ((rc = dalloc(c, &c->d_sys, sizeof(SysDev) * n_sys))) return fail(rc);
   if ((rc = dalloc(c, &c->d_scalar, sizeof(double) * 8))) return fail(rc);
-  int nsm = 0;
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   // Plain form: the O rows are accumulated in their global rows where that lets
   // a second CTA onto the SM (FP64 M^-1 of N = 112 with 1069 parameters: 117
   // against 110 KB a walker; 1024 walkers, a sweep and a measurement 8.4 -> 6.1 ms).

@@ -123,10 +123,21 @@ cudaError_t vmc_launch_expand(const SysDev *h_sys, cudaStream_t st, long long *n
 // (small N, and the mixed form of models with exchange terms, where last bits
 // show in a trajectory; vmc_gj.cuh), double-float (the mixed form's opt-in).
 enum { VMC_INIT_BLOCKED = 0, VMC_INIT_STEPS = 1, VMC_INIT_DF = 2 };
-int vmc_init_form(int precision, int df, int exchange, int n_max);
+// One launch shape per context, so that what is launched is what was sized.
+struct InitPlan {
+  int form = VMC_INIT_BLOCKED;
+  int threads = 0;   // of a CTA
+  size_t smem = 0;   // dynamic shared memory: the largest need of the systems
+};
+// The plan of systems with N[s] electrons per spin on Ns[s] sites, n_work
+// walkers in all, on n_sm SMs; and the bytes one walker's layout takes.  (C
+// linkage: host arithmetic only, checked without a GPU.)
+extern "C" void vmc_init_plan(int precision, int df, int exchange, int n_sys, const int *N,
+                              const int *Ns, int n_work, int n_sm, InitPlan *plan);
+extern "C" size_t vmc_init_smem(int N, int Ns, int form);
 cudaError_t vmc_launch_init(const SysDev *d_sys, const int2 *d_work, int n_work, int *d_ctr,
-                            int precision, int form, int n_max, int only_due, int due_threshold,
-                            size_t smem, cudaStream_t st, long long *nl);
+                            int precision, const InitPlan &plan, int only_due, int due_threshold,
+                            cudaStream_t st, long long *nl);
 cudaError_t vmc_launch_sample(const SysDev *d_sys, const int2 *d_work, int n_work,
                               int *d_work_ctr, int precision, uint64_t seed,
                               int n_first, int n_samples, int sweeps_between,
@@ -160,7 +171,6 @@ cudaError_t vmc_launch_corr_reduce(const double *part, int n_part, const int *cn
 size_t vmc_walker_smem(int precision, int N, int Ns, int acc_len, int H, int kd, int spec_b,
                        int with_lo);
 int vmc_walker_acc_len(int Np);
-size_t vmc_init_smem(int N, int Ns, int form);
 int vmc_sample_occupancy(int precision, size_t smem);
 // the mixed form's 168-register sweep variant (vmc_sweep3.cu)
 int vmc_sample_occupancy_v3(size_t smem);

@@ -31,16 +31,21 @@ __host__ __device__ __forceinline__ size_t minv_bytes(int N, int ldm, int esize)
   return align_up((size_t)N * ldm * esize, 128);
 }
 
-// Shared memory of the from-scratch inverse: the matrix, and the scratch that
-// holds the staged digits of R and, after the elimination, two ints per site.
-// rows: rows of odd stride (step by step, double-float) instead of padded ones.
-__host__ __device__ __forceinline__ size_t init_matrix_bytes(int N, bool rows) {
-  return rows ? align_up((size_t)N * ((N % 2) ? N : N + 1) * sizeof(double), 16)
-              : vmc_gj::gj_matrix_bytes(N);
-}
-__host__ __device__ __forceinline__ size_t init_scratch_bytes(int Ns, bool rows) {
-  const size_t s = align_up(sizeof(int) * (2 * (size_t)Ns + 1), 16);
-  return (rows || s > vmc_gj::GJ_STAGE_BYTES) ? s : vmc_gj::GJ_STAGE_BYTES;
+// Shared memory of the from-scratch inverse: the matrix, the scratch that
+// holds the staged digits of R and, after the elimination, two ints per site,
+// then the electrons' sites and the row order.  rows: rows of odd stride (step
+// by step, double-float) instead of padded ones.
+struct InitLayout {
+  size_t scr, ele, bytes;
+};
+__host__ __device__ __forceinline__ InitLayout init_layout(int N, int Ns, bool rows) {
+  const size_t per_site = align_up(sizeof(int) * (2 * (size_t)Ns + 1), 16);
+  InitLayout l;
+  l.scr = rows ? align_up((size_t)N * ((N % 2) ? N : N + 1) * sizeof(double), 16)
+               : vmc_gj::gj_matrix_bytes(N);
+  l.ele = l.scr + ((rows || per_site > vmc_gj::GJ_STAGE_BYTES) ? per_site : vmc_gj::GJ_STAGE_BYTES);
+  l.bytes = l.ele + sizeof(int) * 3 * (size_t)N;
+  return l;
 }
 
 // ---- TMA bulk copies (cp.async.bulk) with an mbarrier, bounded waits ----
@@ -2312,9 +2317,10 @@ __global__ void __launch_bounds__(NTH, FORM == VMC_INIT_BLOCKED ? 2 : 0)
     double *A = (double *)smem_raw;
     float *Ah = (float *)smem_raw, *Al = Ah + (size_t)N * ldm;
     constexpr bool ROWS = FORM != VMC_INIT_BLOCKED;
-    unsigned char *scr = smem_raw + init_matrix_bytes(N, ROWS);
-    int *ele = (int *)(scr + init_scratch_bytes(Ns, ROWS));   // Ne
-    int *perm = ele + Ne;                                     // N
+    const InitLayout L = init_layout(N, Ns, ROWS);
+    unsigned char *scr = smem_raw + L.scr;
+    int *ele = (int *)(smem_raw + L.ele);   // Ne
+    int *perm = ele + Ne;                   // N
     for (int k = tid; k < Ne; k += nth) ele[k] = S.ele[(size_t)w * Ne + k];
     __syncthreads();
     if constexpr (DF) {
@@ -2558,15 +2564,32 @@ size_t vmc_walker_smem(int precision, int N, int Ns, int acc_len, int H, int kd,
              : walker_layout<float>(N, Ns, acc_len, H, kd, with_lo != 0, true, nullptr, nullptr);
 }
 
-int vmc_init_form(int precision, int df, int exchange, int n_max) {
-  if (precision != 0 && df) return VMC_INIT_DF;
-  return ((precision != 0 && exchange) || n_max <= vmc_gj::GJ_STEPS_MAX_N) ? VMC_INIT_STEPS
-                                                                           : VMC_INIT_BLOCKED;
+extern "C" size_t vmc_init_smem(int N, int Ns, int form) {
+  return init_layout(N, Ns, form != VMC_INIT_BLOCKED).bytes;
 }
 
-size_t vmc_init_smem(int N, int Ns, int form) {
-  const bool rows = form != VMC_INIT_BLOCKED;
-  return init_matrix_bytes(N, rows) + init_scratch_bytes(Ns, rows) + sizeof(int) * 3 * (size_t)N;
+extern "C" void vmc_init_plan(int precision, int df, int exchange, int n_sys, const int *N,
+                              const int *Ns, int n_work, int n_sm, InitPlan *plan) {
+  int n_max = 1;
+  for (int s = 0; s < n_sys; ++s) n_max = N[s] > n_max ? N[s] : n_max;
+  // a walker per SM or fewer: one walker's time is the launch's, and up to N = 48
+  // it is shorter step by step (125 walkers at N = 36, four samples with rebuilds
+  // 1218 -> 1159 us; the gradient of 110 at N = 38 316 -> 308)
+  const bool few = n_work <= n_sm && n_max <= 48;
+  if (precision != 0 && df) plan->form = VMC_INIT_DF;
+  else if ((precision != 0 && exchange) || n_max <= vmc_gj::GJ_STEPS_MAX_N || few) plan->form = VMC_INIT_STEPS;
+  else plan->form = VMC_INIT_BLOCKED;
+  // by panels: up to four walkers per SM take at least NT threads, for the work
+  // per site around the elimination (N = 38 has 96 threads of its own)
+  const int panel_nth = vmc_gj::gj_threads(n_max);
+  plan->threads = plan->form == VMC_INIT_BLOCKED ? (n_work <= 4 * n_sm && panel_nth < NT ? NT : panel_nth)
+                  : plan->form == VMC_INIT_DF    ? NT
+                                                 : vmc_gj::gj_step_threads(n_max);
+  plan->smem = 0;
+  for (int s = 0; s < n_sys; ++s) {
+    const size_t b = vmc_init_smem(N[s], Ns[s], plan->form);
+    plan->smem = b > plan->smem ? b : plan->smem;
+  }
 }
 
 // The mixed form's sweep variant for a shared-memory size: the 168-register
@@ -2632,31 +2655,21 @@ cudaError_t vmc_launch_expand(const SysDev *h_sys, cudaStream_t st, long long *n
 }
 
 cudaError_t vmc_launch_init(const SysDev *d_sys, const int2 *d_work, int n_work, int *d_ctr,
-                            int precision, int form, int n_max, int only_due, int due_threshold,
-                            size_t smem, cudaStream_t st, long long *nl) {
+                            int precision, const InitPlan &plan, int only_due, int due_threshold,
+                            cudaStream_t st, long long *nl) {
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  // a walker per SM or fewer: one walker's time is the launch's, and up to N = 48
-  // it is shorter step by step (125 walkers at N = 36, four samples with rebuilds
-  // 1218 -> 1159 us; the gradient of 110 at N = 38 316 -> 308)
-  if (form == VMC_INIT_BLOCKED && n_work <= nsm && n_max <= 48) form = VMC_INIT_STEPS;
-  // by panels: up to four walkers per SM take at least NT threads, for the work
-  // per site around the elimination (N = 38 has 96 threads of its own)
-  const int panel_nth = vmc_gj::gj_threads(n_max);
-  const int nth = form == VMC_INIT_BLOCKED ? (n_work <= 4 * nsm && panel_nth < NT ? NT : panel_nth)
-                  : form == VMC_INIT_DF    ? NT
-                                           : vmc_gj::gj_step_threads(n_max);
-  const InitKernel kern = init_kernel(precision, form, nth);
+  const InitKernel kern = init_kernel(precision, plan.form, plan.threads);
   int per = 1;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, nth, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, plan.threads, plan.smem);
   if (per < 1) per = 1;
   int grid = nsm * per;
   if (grid > n_work) grid = n_work;
   if (grid < 1) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(d_ctr, 0, sizeof(int), st);
   if (e) return e;
-  kern<<<grid, nth, smem, st>>>(d_sys, d_work, n_work, d_ctr, only_due, due_threshold);
+  kern<<<grid, plan.threads, plan.smem, st>>>(d_sys, d_work, n_work, d_ctr, only_due, due_threshold);
   ++*nl;
   return cudaGetLastError();
 }
