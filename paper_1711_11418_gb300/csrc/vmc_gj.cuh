@@ -666,6 +666,47 @@ __device__ __forceinline__ void gj_steps(double *A, int lda, int N, int *perm, G
   __syncthreads();
 }
 
+// The inverse by panels of the matrix entry(n, m), which A holds already (padded,
+// gj_at); if it is close to singular, step by step after all, from entry() again,
+// in rows of ld = N or N + 1 (odd).  stage: the staged digits' space (16-byte
+// aligned), perm: N ints, red: a word per warp.  Every thread returns the same.
+struct GJResult {
+  int bad, sign;
+  double logdet, pmin, pmax;
+  bool steps;   // the inverse's entry (k, c) is A[k ld + c], else gj_inverse_at
+};
+template <typename Entry>
+__device__ __forceinline__ GJResult gj_invert_guarded(double *A, uint32_t *stage, int N, int *perm,
+                                                      GJShared &g, double *red, Entry entry) {
+  const int tid = threadIdx.x, nwarps = blockDim.x >> 5, ld = (N % 2) ? N : N + 1;
+  gj_invert(A, stage, N, g);
+  GJResult r = {g.bad, g.sign, g.logdet, g.pmin, g.pmax, false};
+  double amax = 0.0;
+  if (!r.bad)   // the inverse's entries, in the order they are stored
+    for (int i = tid >> 5; i < N; i += nwarps)
+      for (int q = tid & 31; q < N; q += 32) amax = fmax(amax, fabs(A[gj_at(i, q, gj_pad(N))]));
+  for (int o = 16; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+  if ((tid & 31) == 0) red[tid >> 5] = amax;
+  __syncthreads();
+  for (int q = 0; q < nwarps; ++q) amax = fmax(amax, red[q]);
+  r.steps = r.bad || !(amax * r.pmax <= GJ_BLOCKED_COND);
+  __syncthreads();
+  if (r.steps) {
+    GJSteps &g2 = *(GJSteps *)((unsigned char *)stage + GJ_REDO_OFFSET);
+    for (int q = tid; q < N * N; q += blockDim.x) {
+      const int n = q / N, m = q - n * N;
+      A[n * ld + m] = entry(n, m);
+    }
+    __syncthreads();
+    gj_steps<0>(A, ld, N, perm, g2);
+    r.bad = g2.bad;
+    r.sign = g2.sign;
+    r.logdet = g2.logdet;
+    r.pmin = g2.pmin;
+    r.pmax = g2.pmax;
+  }
+  return r;
+}
 
 inline int gj_step_threads(int n_max) { return n_max > 112 ? 32 * ST_WARPS : 128; }
 

@@ -363,10 +363,6 @@ __device__ void proj_exchange_update(T *Mg, int N, int n, int m, const T *w, con
 // ---------------------------------------------------------------------------
 // From-scratch inverses: one CTA per (walker, operation)
 // ---------------------------------------------------------------------------
-// M_g gathered in FP64, Gauss-Jordan in shared memory; M_g^-1 written in the
-// context's precision; log|A_g| and the sign of A_g = sigma_g det M_g kept
-// for the shares (k_proj_shares).  With only_due, walkers whose accepted-move
-// count has not reached due_threshold are skipped.
 // FP64 inverses by panels above GJ_STEPS_MAX_N, the others and the mixed form's
 // FP32 ones step by step (vmc_gj.cuh has the reasons).
 static bool build_by_panels(int precision, int n_max) {
@@ -379,6 +375,10 @@ __host__ __device__ inline size_t build_matrix_bytes(bool panels, int N) {
                 : pal((size_t)N * ((N % 2) ? N : N + 1) * sizeof(double));
 }
 
+// M_g gathered in FP64, Gauss-Jordan in shared memory; M_g^-1 written in the
+// context's precision; log|A_g| and the sign of A_g = sigma_g det M_g kept
+// for the shares (k_proj_shares).  With only_due, walkers whose accepted-move
+// count has not reached due_threshold are skipped.
 template <typename T, bool PANELS, int NTH>   // NTH as of k_init
 __global__ void __launch_bounds__(NTH, PANELS ? 2 : 0)
     k_proj_build(const SysDev *systems, const int2 *work, int n_work, int Ng, int only_due,
@@ -388,6 +388,7 @@ __global__ void __launch_bounds__(NTH, PANELS ? 2 : 0)
   using Scratch = typename std::conditional<PANELS, vmc_gj::GJShared, vmc_gj::GJSteps>::type;
   __shared__ Scratch gs;
   __shared__ int sgm;
+  __shared__ double red[NTH / 32];
   const int tid = threadIdx.x, nth = PANELS ? blockDim.x : NTH;
   for (long long item = blockIdx.x; item < (long long)n_work * Ng; item += gridDim.x) {
     __syncthreads();
@@ -415,25 +416,40 @@ __global__ void __launch_bounds__(NTH, PANELS ? 2 : 0)
       if (tid == 0) sgm = (neg & 1) ? -1 : 1;
     }
     __syncthreads();
+    auto entry = [&](int n, int m) -> double { return S.f64[(size_t)gsite[n] * Ns + gsite[N + m]]; };
     for (int q = tid; q < P * P; q += nth) {
       const int n = q / P, m = q - n * P;
-      const double f = (n < N && m < N) ? S.f64[(size_t)gsite[n] * Ns + gsite[N + m]]
-                                        : (n == m ? 1.0 : 0.0);
-      A[PANELS ? vmc_gj::gj_at(n, m, P) : n * ldm + m] = f;
+      A[PANELS ? vmc_gj::gj_at(n, m, P) : n * ldm + m] =
+          (n < N && m < N) ? entry(n, m) : (n == m ? 1.0 : 0.0);
     }
     __syncthreads();
-    if constexpr (PANELS) vmc_gj::gj_invert(A, stage, N, gs);
-    else vmc_gj::gj_steps<NTH>(A, ldm, N, gsite + Ne, gs);
+    int bad, sign;
+    double logdet;
+    bool steps = true;
+    if constexpr (PANELS) {
+      const vmc_gj::GJResult r = vmc_gj::gj_invert_guarded(A, stage, N, gsite + Ne, gs, red, entry);
+      bad = r.bad;
+      sign = r.sign;
+      logdet = r.logdet;
+      steps = r.steps;
+    } else {
+      vmc_gj::gj_steps<NTH>(A, ldm, N, gsite + Ne, gs);
+      bad = gs.bad;
+      sign = gs.sign;
+      logdet = gs.logdet;
+    }
     T *dst = proj_minv<T>(S, w, g);
     for (int q = tid; q < N * N; q += nth) {
       const int n = q / N, m = q - n * N;
-      if constexpr (PANELS) dst[q] = gs.bad ? (T)0 : (T)vmc_gj::gj_inverse_at(A, N, n, m, gs);
-      else dst[q] = gs.bad ? (T)0 : (T)A[n * ldm + m];
+      double a;
+      if constexpr (PANELS) a = steps ? A[n * ldm + m] : vmc_gj::gj_inverse_at(A, N, n, m, gs);
+      else a = A[n * ldm + m];
+      dst[q] = bad ? (T)0 : (T)a;
     }
     if (tid == 0) {
       const size_t k = (size_t)w * Ng + g;
-      S.plog[k] = gs.bad ? -INFINITY : gs.logdet;
-      S.psign[k] = gs.bad ? 0 : gs.sign * sgm;
+      S.plog[k] = bad ? -INFINITY : logdet;
+      S.psign[k] = bad ? 0 : sign * sgm;
     }
   }
 }

@@ -2323,59 +2323,39 @@ __global__ void __launch_bounds__(NTH, FORM == VMC_INIT_BLOCKED ? 2 : 0)
     int *perm = ele + Ne;                   // N
     for (int k = tid; k < Ne; k += nth) ele[k] = S.ele[(size_t)w * Ne + k];
     __syncthreads();
-    if constexpr (DF) {
-      for (int q = tid; q < N * N; q += nth) {
-        const int n = q / N, m = q - n * N;
-        df_split(S.f64[(size_t)ele[n] * Ns + ele[N + m]], Ah[n * ldm + m], Al[n * ldm + m]);
-      }
-      __syncthreads();
-      gj_invert_df(Ah, Al, ldm, N, perm, gs);
-    } else if constexpr (FORM == VMC_INIT_STEPS) {
-      for (int q = tid; q < N * N; q += nth) {
-        const int n = q / N, m = q - n * N;
-        A[n * ldm + m] = S.f64[(size_t)ele[n] * Ns + ele[N + m]];
-      }
-      __syncthreads();
-      vmc_gj::gj_steps<NTH>(A, ldm, N, perm, gs);
-    } else {
+    int g_bad, g_sign;
+    double g_logdet, g_pmin, g_pmax;
+    bool redone = false;   // by panels: close to singular, eliminated again step by step
+    auto entry = [&](int n, int m) -> double { return S.f64[(size_t)ele[n] * Ns + ele[N + m]]; };
+    if constexpr (FORM == VMC_INIT_BLOCKED) {
       const int P = vmc_gj::gj_pad(N);
       for (int q = tid; q < P * P; q += nth) {
         const int n = q / P, m = q - n * P;
-        A[vmc_gj::gj_at(n, m, P)] = (n < N && m < N) ? S.f64[(size_t)ele[n] * Ns + ele[N + m]]
-                                                     : (n == m ? 1.0 : 0.0);
+        A[vmc_gj::gj_at(n, m, P)] = (n < N && m < N) ? entry(n, m) : (n == m ? 1.0 : 0.0);
       }
       __syncthreads();
-      vmc_gj::gj_invert(A, (uint32_t *)scr, N, gs);
-    }
-    int g_bad = gs.bad, g_sign = gs.sign;
-    double g_logdet = gs.logdet, g_pmin = gs.pmin, g_pmax = gs.pmax;
-    bool redone = false;   // by panels: close to singular, eliminated again step by step
-    if constexpr (FORM == VMC_INIT_BLOCKED) {
-      double amax = 0.0;
-      if (!g_bad)   // the inverse's entries, in the order they are stored
-        for (int r = tid >> 5; r < N; r += nth / 32)
-          for (int q = tid & 31; q < N; q += 32)
-            amax = fmax(amax, fabs(A[vmc_gj::gj_at(r, q, vmc_gj::gj_pad(N))]));
-      for (int o = 16; o > 0; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-      if ((tid & 31) == 0) red_a[tid >> 5] = amax;
-      __syncthreads();
-      for (int q = 0; q < nth / 32; ++q) amax = fmax(amax, red_a[q]);
-      redone = g_bad || !(amax * g_pmax <= vmc_gj::GJ_BLOCKED_COND);
-      __syncthreads();
-      if (redone) {
-        vmc_gj::GJSteps &g2 = *(vmc_gj::GJSteps *)(scr + vmc_gj::GJ_REDO_OFFSET);
-        for (int q = tid; q < N * N; q += nth) {
-          const int n = q / N, m = q - n * N;
-          A[n * ldm + m] = S.f64[(size_t)ele[n] * Ns + ele[N + m]];
-        }
-        __syncthreads();
-        vmc_gj::gj_steps<0>(A, ldm, N, perm, g2);
-        g_bad = g2.bad;
-        g_sign = g2.sign;
-        g_logdet = g2.logdet;
-        g_pmin = g2.pmin;
-        g_pmax = g2.pmax;
+      const vmc_gj::GJResult r =
+          vmc_gj::gj_invert_guarded(A, (uint32_t *)scr, N, perm, gs, red_a, entry);
+      g_bad = r.bad;
+      g_sign = r.sign;
+      g_logdet = r.logdet;
+      g_pmin = r.pmin;
+      g_pmax = r.pmax;
+      redone = r.steps;
+    } else {
+      for (int q = tid; q < N * N; q += nth) {
+        const int n = q / N, m = q - n * N;
+        if constexpr (DF) df_split(entry(n, m), Ah[n * ldm + m], Al[n * ldm + m]);
+        else A[n * ldm + m] = entry(n, m);
       }
+      __syncthreads();
+      if constexpr (DF) gj_invert_df(Ah, Al, ldm, N, perm, gs);
+      else vmc_gj::gj_steps<NTH>(A, ldm, N, perm, gs);
+      g_bad = gs.bad;
+      g_sign = gs.sign;
+      g_logdet = gs.logdet;
+      g_pmin = gs.pmin;
+      g_pmax = gs.pmax;
     }
     // the fresh inverse's entry (r, c) (FP64 value)
     auto fresh_at = [&](int r, int c) -> double {
