@@ -116,6 +116,22 @@ __device__ __forceinline__ int vmc_mulhi(uint32_t r, int n) {
   return (int)(((unsigned long long)r * (unsigned long long)n) >> 32);
 }
 
+// Lets a kernel take `need` bytes of dynamic shared memory (an error if it
+// cannot).  The limit belongs to the kernel, not to the context: it is the
+// largest possible one on every call, so that contexts of other sizes and other
+// threads' calls do not lower it.
+inline cudaError_t vmc_smem_limit(const void *kernel, size_t need) {
+  int dev = 0, optin = 0;
+  cudaFuncAttributes at;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev))) return e;
+  if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev))) return e;
+  if ((e = cudaFuncGetAttributes(&at, kernel))) return e;
+  if (need + at.sharedSizeBytes > (size_t)optin) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              optin - (int)at.sharedSizeBytes);
+}
+
 // ---- launch wrappers (defined in vmc_walker.cu / vmc_sr.cu) ----
 // All return cudaError_t from the launch; they count launches in *n_launch.
 cudaError_t vmc_launch_expand(const SysDev *h_sys, cudaStream_t st, long long *n_launch);

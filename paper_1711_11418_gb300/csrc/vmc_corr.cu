@@ -457,10 +457,7 @@ cudaError_t vmc_corr_shape(int precision, int N, int Ns, int W, CorrShape *out) 
   out->rows = (int)rows;
   out->smem = precision == 0 ? corr_layout<double>(N, Ns, (int)rows, nullptr, nullptr)
                              : corr_layout<float>(N, Ns, (int)rows, nullptr, nullptr);
-  // the same limit on every call, so calls of several threads do not undo each other's
-  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                optin - (int)stat)))
-    return e;
+  if ((e = vmc_smem_limit((const void *)kern, out->smem))) return e;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, CNT, out->smem))) return e;
   if (per < 1) per = 1;
   const long long grid = (long long)nsm * per;

@@ -400,7 +400,7 @@ static cudaError_t lz_config(int precision, int Ns, int N, LzKernel *k, size_t *
   const bool vs = precision == 0 ? lz_vec_smem<double>(Ns, N) : lz_vec_smem<float>(Ns, N);
   *k = lz_kernel(precision, vs);
   *smem = precision == 0 ? lz_smem<double>(Ns, N, vs) : lz_smem<float>(Ns, N, vs);
-  cudaError_t e = cudaFuncSetAttribute(*k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
+  cudaError_t e = vmc_smem_limit((const void *)*k, *smem);
   if (e) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, *k, LZ_NT, *smem);
 }

@@ -1014,15 +1014,13 @@ static BuildKernel build_kernel(int precision, bool panels, int nth) {
 
 cudaError_t vmc_proj_set_smem(size_t s_sample, size_t s_build) {
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(k_proj_sample<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_sample))) return e;
-  if ((e = cudaFuncSetAttribute(k_proj_sample<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_sample))) return e;
-  if ((e = cudaFuncSetAttribute(k_proj_eval<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_sample))) return e;
-  if ((e = cudaFuncSetAttribute(k_proj_eval<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_sample))) return e;
+  if ((e = vmc_smem_limit((const void *)k_proj_sample<double>, s_sample))) return e;
+  if ((e = vmc_smem_limit((const void *)k_proj_sample<float>, s_sample))) return e;
+  if ((e = vmc_smem_limit((const void *)k_proj_eval<double>, s_sample))) return e;
+  if ((e = vmc_smem_limit((const void *)k_proj_eval<float>, s_sample))) return e;
   for (int q = 0; q < 3; ++q)   // FP64 by panels, FP64 and FP32 step by step
     for (int nth : {NT, vmc_gj::MAX_THREADS})
-      if ((e = cudaFuncSetAttribute(build_kernel(q == 2, q == 0, nth),
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s_build)))
-        return e;
+      if ((e = vmc_smem_limit((const void *)build_kernel(q == 2, q == 0, nth), s_build))) return e;
   return cudaSuccess;
 }
 

@@ -2612,9 +2612,7 @@ cudaError_t vmc_walker_set_smem_limits(size_t s64, size_t s32, size_t sinit) {
   for (int form : {VMC_INIT_BLOCKED, VMC_INIT_STEPS, VMC_INIT_DF})
     for (int prec = 0; prec < 2; ++prec)
       for (int nth : {NT, vmc_gj::MAX_THREADS})
-        if ((e = cudaFuncSetAttribute(init_kernel(prec, form, nth),
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sinit)))
-          return e;
+        if ((e = vmc_smem_limit((const void *)init_kernel(prec, form, nth), sinit))) return e;
   return cudaSuccess;
 }
 
