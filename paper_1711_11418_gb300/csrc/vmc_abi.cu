@@ -461,7 +461,7 @@ int sr_alloc(vmc_ctx *c, SysHost &s, bool need_S, bool need_ir = false) {
       // kernel builds S otherwise)
       unsigned char *dg = nullptr;
       int *em = nullptr;
-      if (dalloc(c, &em, sizeof(int) * s.Np) == VMC_OK &&
+      if (dalloc(c, &em, sizeof(int) * (s.Np + 1)) == VMC_OK &&
           dalloc(c, &dg, vmc_sr_digits_bytes(rows_cap, s.Np)) == VMC_OK) {
         s.sr.digits = dg;
         s.sr.emax = em;

@@ -253,7 +253,7 @@ struct SrWork {
   int ir_iter;
   double ir_eps;
   unsigned char *digits;       // plain form: a slab of samples as digits (vmc_sr_digits.cu), or null
-  int *emax;                   // [Np] exponents of the centred columns
+  int *emax;                   // [Np] exponents of the centred columns, [1] some are not finite
   int stall;                   // test hook: CTA 0 of the next tensor-core S build waits on a
                                // barrier nothing arrives on (then no copy or MMA is issued)
 };

@@ -13,6 +13,7 @@
 //               samples at a time; every KC = 128 samples (7 x 128 x 2^14 <
 //               2^24: the sums are exact up to there) the eight sums become one
 //               FP64 number, added to the lane's entries in FP64.
+//   k_syrk_nonfinite  the entries of columns with infinities or NaNs
 //
 // What is left out is below 2^-56 of a column's largest entry, at most the
 // FP64 rounding of the entries themselves for all but the smallest ones.
@@ -38,6 +39,7 @@ constexpr int ST = 3;                // stages
 constexpr int BLK = 512;             // bytes of one digit of a 16 x 16 block
 constexpr int STAGE = 2 * (TS / 16) * NDIG * (KS / 16) * BLK;   // both operands
 constexpr int THREADS = 512;
+constexpr int NONFINITE = 0x7ff;     // exponent of a column with an infinity or a NaN
 
 __global__ void k_dig_max(const double *O, int ldO, int rows, int Np, const double *obar, int chunk,
                           int *emax) {
@@ -55,6 +57,7 @@ __global__ void k_dig_max(const double *O, int ldO, int rows, int Np, const doub
   if (threadIdx.y == 0 && c < Np) {
     for (int q = 1; q < 8; ++q) e = max(e, sh[q][threadIdx.x]);
     atomicMax(emax + c, e);
+    if (e == NONFINITE) emax[Np] = 1;   // the columns have one
   }
 }
 
@@ -196,6 +199,24 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
 }
 
+// Fixed point knows no infinities and NaNs: the entries of S of the columns that
+// have one are summed in FP64 here, as IEEE arithmetic gives them (a row of S
+// per CTA; returns at once where there is no such column).
+__global__ void __launch_bounds__(256) k_syrk_nonfinite(const double *O, int ldO, int rows, int Np,
+                                                        const double *obar, const int *emax,
+                                                        double scale, double *S) {
+  if (!emax[Np]) return;
+  const int i = blockIdx.x;
+  const bool all = emax[i] == NONFINITE;
+  for (int j = i + threadIdx.x; j < Np; j += blockDim.x) {
+    if (!all && emax[j] != NONFINITE) continue;
+    double s = 0.0;
+    for (int r = 0; r < rows; ++r)
+      s += (O[(size_t)r * ldO + i] - obar[i]) * (O[(size_t)r * ldO + j] - obar[j]);
+    S[(size_t)i * Np + j] = s * scale;
+  }
+}
+
 // Digit blocks of 16 samples per slab: at most 1 GiB of digits.
 constexpr size_t SLAB_BYTES = 1ull << 30;
 int pad_blocks(int Np) { return (Np + TS - 1) / TS * (TS / 16); }
@@ -214,11 +235,11 @@ size_t vmc_sr_digits_bytes(int rows, int Np) {
 }
 
 // S (upper triangle; zeroed by the caller) += (1/rows) (O - o)^T (O - o) of the
-// FP64 samples; digits: vmc_sr_digits_bytes(rows, Np), emax: Np ints.
+// FP64 samples; digits: vmc_sr_digits_bytes(rows, Np), emax: Np + 1 ints.
 cudaError_t vmc_sr_syrk_digits(const SrWork &w, unsigned char *digits, int *emax, cudaStream_t st,
                                long long *nl) {
   const double *O = (const double *)w.O;
-  cudaError_t e = cudaMemsetAsync(emax, 0, sizeof(int) * w.Np, st);
+  cudaError_t e = cudaMemsetAsync(emax, 0, sizeof(int) * (w.Np + 1), st);
   if (e) return e;
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
@@ -249,6 +270,7 @@ cudaError_t vmc_sr_syrk_digits(const SrWork &w, unsigned char *digits, int *emax
                                                                  w.Np, emax, 1.0 / w.rows, w.S);
     *nl += 2;
   }
-  *nl += 1;
+  k_syrk_nonfinite<<<w.Np, 256, 0, st>>>(O, w.ldO, w.rows, w.Np, w.obar, emax, 1.0 / w.rows, w.S);
+  *nl += 2;
   return cudaGetLastError();
 }
