@@ -436,7 +436,7 @@ int sr_alloc(vmc_ctx *c, SysHost &s, bool need_S, bool need_ir = false) {
     CK(dalloc(c, &w.scal, sizeof(double) * 8));
     CK(dalloc(c, &w.info, sizeof(int) * 4));
     CK(dalloc(c, &w.dblk, sizeof(double) * 32 * 32));
-    CK(dalloc(c, &w.dinv, sizeof(double) * 32 * (size_t)((Np + 31) / 32 * 32)));
+    CK(dalloc(c, &w.dinv, sizeof(double) * (size_t)Np));
     CK(dalloc(c, &w.vf, sizeof(float) * Np));
     CK(dalloc(c, &w.tf, sizeof(float) * rows_cap));
     CK(dalloc(c, &w.dpart, sizeof(double) * 512));

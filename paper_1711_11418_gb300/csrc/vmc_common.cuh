@@ -238,7 +238,7 @@ struct SrWork {
   double *scal;                // device scalars
   int *info;                   // device status
   double *dblk;                // [32*32] factored diagonal block in flight (Cholesky)
-  double *dinv;                // [ceil(Np/32)*32*32] inverses of the diagonal blocks of L
+  double *dinv;                // [Np] reciprocals of the diagonal of L
   double *part;                // column-reduction partials [2 * vmc_colreduce_parts(rows, Np) * Np]
   float *vf, *tf;              // FP32 copies of the SR-CG vectors (mixed form) [Np], [rows]
   double *dpart;               // dot-product partials [512]

@@ -279,13 +279,16 @@ __global__ void k_mirror_shift(double *S, int Np, double shift_rel, double shift
 
 // Blocked right-looking Cholesky (lower triangle in place), panels of CB
 // columns.  Per panel: k_chol_panel factors the diagonal block, L_jj L_jj^T,
-// forms L_jj^-1 and with it the panel below (L_ij = A_ij L_jj^-T) and the
-// panel's part of the forward solution L z = g; k_syrk_trailing updates the
-// trailing lower triangle (A -= L L^T) in 32x32 tiles and the rest of the
-// right-hand side.  What bounds it: the chain of n pivots (about 1000 clocks
-// each: a reciprocal, a column, a barrier, eight multiply-adds on a pipe that
-// takes 64 clocks for a warp's) and the FP64 pipe for n^3 / 3 multiply-adds.
-// n = 1069: panels 2.37 -> 1.04 ms, both triangular solves 1.32 -> 0.16 ms.
+// and forms the panel below (L_ij = A_ij L_jj^-T) and its part of the forward
+// solution L z = g by substitution; k_syrk_trailing updates the trailing lower
+// triangle (A -= L L^T) in 32x32 tiles and the rest of the right-hand side.
+// What bounds it: the chain of n pivots (a reciprocal, a column, a barrier, up
+// to eight multiply-adds on a pipe that takes 64 clocks for a warp's) and the
+// FP64 pipe for n^3 / 3 multiply-adds.  Products with the diagonal blocks'
+// inverses are shorter chains, but their residual grows with the condition of
+// the block: |S x - g| at neighbouring columns that are nearly alike, cond(S) =
+// 1e10, was 2000 to 6000 times that of substitution, and past 1e13 the
+// factorisation broke down.
 constexpr int CB = 32;
 constexpr int PT = 128;    // threads of k_chol_panel
 
@@ -302,35 +305,37 @@ __device__ __forceinline__ double fast_recip(double x) {
 
 // Panel step.  Every CTA factors the nb x nb diagonal block redundantly, lane =
 // row, warp w the columns w, w + 4, ...: elimination without square roots
-// (A = L1 D L1^T, L1 unit) applied to the identity beside it, which gives
-// W1 = L1^-1; L_jj = L1 D^1/2 and W = D^-1/2 W1 = L_jj^-1.  Then four threads
-// to a row form X_i = A_i W^T for CB rows below.  CTA 0 records the first
-// non-positive pivot in *info (1-based), stores W, the panel of the forward
-// solution z = W y, and the factored block: straight into A when it is the only
-// CTA, else into dblk, from where the trailing update copies it (another CTA
-// may still be reading the block).
+// (A = L1 D L1^T, L1 unit), L_jj = L1 D^1/2.  All CTAs but the last then solve
+// X L_jj^T = A_i for CB rows below, four threads to a row, thread q the columns
+// q, q + 4, ...: column c is finished and taken out of the later ones.  The last
+// CTA records the first non-positive pivot in *info (1-based), stores 1 / L_kk
+// (dinv) and the panel of the forward solution z, and the factored block: into A
+// when it is the only CTA, else into dblk, from where the trailing update copies
+// it (another CTA may still be reading the block).
 __global__ void __launch_bounds__(PT) k_chol_panel(double *A, int n, int j0, int nb, int *info,
-                                                   double *dblk, double *Wout, const double *y,
+                                                   double *dblk, double *dinv, const double *y,
                                                    double *z) {
-  __shared__ double Ls[CB][CB + 1], Ws[CB][CB + 1];
+  __shared__ double Ls[CB][CB + 1];
   __shared__ double mcol[2][CB], acol[2][CB];   // multipliers, column before scaling
   __shared__ double dg[CB], sq[CB], rs[CB];
   __shared__ int bad_sh;
   const int tid = threadIdx.x, r = tid & 31, w = tid >> 5;
+  const bool last = blockIdx.x == gridDim.x - 1;
   if (tid == 0) bad_sh = 0;
-  double a[CB / 4], v[CB / 4];
+  double a[CB / 4];
 #pragma unroll
   for (int j = 0; j < CB / 4; ++j) {
     const int c = w + 4 * j;
     a[j] = (r < nb && c <= r) ? A[(size_t)(j0 + r) * n + j0 + c] : (r == c ? 1.0 : 0.0);
-    v[j] = (r == c) ? 1.0 : 0.0;
   }
-  // this thread's row of the panel below, fetched while the block is factored
+  // this thread's entries of the panel below, fetched while the block is factored
+  const int q = tid & 3;
   const int i = j0 + nb + blockIdx.x * CB + (tid >> 2);
-  const bool row_ok = blockIdx.x * CB + (tid >> 2) < n - j0 - nb;
-  double x[CB];
+  const bool row_ok = !last && i < n;
+  double x[CB / 4];
 #pragma unroll
-  for (int l = 0; l < CB; ++l) x[l] = (row_ok && l < nb) ? A[(size_t)i * n + j0 + l] : 0.0;
+  for (int j = 0; j < CB / 4; ++j)
+    x[j] = (row_ok && q + 4 * j < nb) ? A[(size_t)i * n + j0 + q + 4 * j] : 0.0;
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < CB; ++k) {
@@ -355,11 +360,6 @@ __global__ void __launch_bounds__(PT) k_chol_panel(double *A, int n, int j0, int
       const int c = w + 4 * j;
       if (c > k) a[j] = fma(-m, acol[b][c], a[j]);   // rows r >= c matter
     }
-#pragma unroll
-    for (int j = 0; j <= (k >> 2); ++j) {
-      const double vk = __shfl_sync(0xffffffffu, v[j], k);
-      if (w + 4 * j <= k) v[j] = fma(-m, vk, v[j]);
-    }
   }
   if (w == 0) {
     const double d = dg[r];
@@ -372,14 +372,12 @@ __global__ void __launch_bounds__(PT) k_chol_panel(double *A, int n, int j0, int
   for (int j = 0; j < CB / 4; ++j) {
     const int c = w + 4 * j;
     Ls[r][c] = c <= r ? a[j] * sq[c] : 0.0;
-    Ws[r][c] = c <= r ? v[j] * rs[r] : 0.0;
   }
   __syncthreads();
-  if (blockIdx.x == 0) {
+  if (last) {
     const bool direct = gridDim.x == 1;
-    for (int q = tid; q < CB * CB; q += PT) {
-      const int rr = q / CB, c = q % CB;
-      Wout[q] = Ws[rr][c];
+    for (int p = tid; p < CB * CB; p += PT) {
+      const int rr = p / CB, c = p % CB;
       if (rr < nb && c <= rr) {
         if (direct) A[(size_t)(j0 + rr) * n + j0 + c] = Ls[rr][c];
         else dblk[rr * nb + c] = Ls[rr][c];
@@ -387,38 +385,42 @@ __global__ void __launch_bounds__(PT) k_chol_panel(double *A, int n, int j0, int
     }
     if (tid == 0 && bad_sh && *info == 0) *info = j0 + bad_sh;
     if (w == 3) {
-      double s0 = 0.0, s1 = 0.0;
-      for (int l = 0; l < nb; l += 2) {
-        s0 = fma(Ws[r][l], y[j0 + l], s0);
-        if (l + 1 < nb) s1 = fma(Ws[r][l + 1], y[j0 + l + 1], s1);
+      double v = r < nb ? y[j0 + r] : 0.0;
+#pragma unroll
+      for (int k = 0; k < CB; ++k) {
+        const double zk = __shfl_sync(0xffffffffu, v, k) * rs[k];
+        if (r == k) v = zk;
+        else if (r > k) v = fma(-Ls[r][k], zk, v);
       }
-      if (r < nb) z[j0 + r] = s0 + s1;
+      if (r < nb) {
+        z[j0 + r] = v;
+        dinv[j0 + r] = rs[r];
+      }
     }
+    return;
   }
-  if (!row_ok) return;
-  const int q = tid & 3;
 #pragma unroll
-  for (int j = 0; j < CB / 4; ++j) {
-    const int c = q + 4 * j;
-    double s0 = 0.0, s1 = 0.0;
+  for (int c = 0; c < CB; ++c) {
+    const double xc = __shfl_sync(0xffffffffu, x[c >> 2], (tid & 28) | (c & 3)) * rs[c];
+    if (q == (c & 3)) x[c >> 2] = xc;
 #pragma unroll
-    for (int l = 0; l < 4 * j + 4; l += 2) {   // W is lower triangular: l <= c
-      s0 = fma(x[l], Ws[c][l], s0);
-      s1 = fma(x[l + 1], Ws[c][l + 1], s1);
-    }
-    if (c < nb) A[(size_t)i * n + j0 + c] = s0 + s1;
+    for (int j = c >> 2; j < CB / 4; ++j)
+      if (q + 4 * j > c) x[j] = fma(-xc, Ls[q + 4 * j][c], x[j]);
   }
+#pragma unroll
+  for (int j = 0; j < CB / 4; ++j)
+    if (row_ok && q + 4 * j < nb) A[(size_t)i * n + j0 + q + 4 * j] = x[j];
 }
 
 // Trailing update A[i][k] -= sum_l L[i][j0+l] L[k][j0+l] for j1 <= k <= i < n
 // (j1 = j0 + nb): one 32x32 lower tile per CTA, tile (bi, bj) with bj <= bi
-// decoded from the linear block index.  With copy_diag, CTA 0 also stores
-// the factored diagonal block from dblk (no CTA here reads that block).
+// decoded from the linear block index.  CTA 0 also stores the factored diagonal
+// block from dblk (no CTA here reads that block).
 // CTAs from n_tiles on take the panel out of the right-hand side instead:
 // y_k -= sum_l L_{k,j0+l} z_{j0+l}, 256 rows k each.
 __global__ void __launch_bounds__(256) k_syrk_trailing(double *A, int n, int j0, int nb,
-                                                       int copy_diag, const double *dblk,
-                                                       int n_tiles, double *y, const double *z) {
+                                                       const double *dblk, int n_tiles, double *y,
+                                                       const double *z) {
   const int j1 = j0 + nb;
   if (blockIdx.x >= n_tiles) {
     __shared__ double zp[CB];
@@ -437,7 +439,7 @@ __global__ void __launch_bounds__(256) k_syrk_trailing(double *A, int n, int j0,
     }
     return;
   }
-  if (copy_diag && blockIdx.x == 0)
+  if (blockIdx.x == 0)
     for (int q = threadIdx.x; q < nb * nb; q += 256) {
       const int r = q / nb, c = q % nb;
       if (c <= r) A[(size_t)(j0 + r) * n + j0 + c] = dblk[q];
@@ -476,40 +478,46 @@ __global__ void __launch_bounds__(256) k_syrk_trailing(double *A, int n, int j0,
 }
 
 // Backward solve L^T x = z, one launch per panel of CB unknowns, last first:
-// every CTA forms x_p = W^T z_p (W = L_pp^-1 of the factorisation; eight warps
-// share the sums), then takes the panel out of its share of the entries above,
-// z_i -= sum_l L_{p0+l,i} x_{p0+l} for i < p0 (thread per entry).  z is read
-// and x written to another vector, so no CTA reads what another one writes.
+// every CTA solves L_pp^T x_p = z_p by substitution (a lane per unknown), then
+// takes the panel out of its share of the entries above, z_i -= sum_l L_{p0+l,i}
+// x_{p0+l} for i < p0 (thread per entry).  z is read and x written to another
+// vector, so no CTA reads what another one writes.
 constexpr int SV_COLS = 256;
 
 __global__ void __launch_bounds__(SV_COLS) k_trsv_back(const double *L, int n, int p0,
-                                                       const double *W, double *z, double *x) {
-  __shared__ double part[8][CB], xp[CB];
+                                                       const double *dinv, double *z, double *x) {
+  __shared__ double Ls[CB][CB + 1], xp[CB];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nb = min(CB, n - p0);
-  double s = 0.0;
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int rr = warp * 4 + u;
-    if (rr < nb) s = fma(W[rr * CB + lane], z[p0 + rr], s);   // W[rr][lane] = 0 for rr < lane
+  for (int u = 0; u < CB / 8; ++u) {
+    const int r = warp + 8 * u;
+    Ls[r][lane] = (r < nb && lane < r) ? L[(size_t)(p0 + r) * n + p0 + lane] : 0.0;
   }
-  part[warp][lane] = s;
+  const int i = blockIdx.x * SV_COLS + tid;
+  double col[CB];   // this thread's column of the panel, fetched while x_p is formed
+#pragma unroll
+  for (int l = 0; l < CB; ++l) col[l] = (i < p0 && l < nb) ? L[(size_t)(p0 + l) * n + i] : 0.0;
   __syncthreads();
   if (warp == 0) {
-    double t = part[0][lane];
+    double v = lane < nb ? z[p0 + lane] : 0.0;
+    const double rd = lane < nb ? dinv[p0 + lane] : 0.0;
 #pragma unroll
-    for (int k = 1; k < 8; ++k) t += part[k][lane];
-    xp[lane] = lane < nb ? t : 0.0;
-    if (blockIdx.x == 0 && lane < nb) x[p0 + lane] = t;
+    for (int k = CB - 1; k >= 0; --k) {
+      const double xk = __shfl_sync(0xffffffffu, v * rd, k);
+      if (lane == k) v = xk;
+      else if (lane < k) v = fma(-Ls[k][lane], xk, v);
+    }
+    xp[lane] = lane < nb ? v : 0.0;
+    if (blockIdx.x == 0 && lane < nb) x[p0 + lane] = v;
   }
   __syncthreads();
-  const int i = blockIdx.x * SV_COLS + tid;
   if (i < p0) {
     double s0 = 0.0, s1 = 0.0;
-#pragma unroll 8
+#pragma unroll
     for (int l = 0; l < CB; l += 2) {
-      if (l < nb) s0 = fma(L[(size_t)(p0 + l) * n + i], xp[l], s0);
-      if (l + 1 < nb) s1 = fma(L[(size_t)(p0 + l + 1) * n + i], xp[l + 1], s1);
+      s0 = fma(col[l], xp[l], s0);
+      s1 = fma(col[l + 1], xp[l + 1], s1);
     }
     z[i] -= s0 + s1;
   }
@@ -683,18 +691,16 @@ static void chol_sequence(const SrWork &w, cudaStream_t st) {
   for (int j0 = 0; j0 < n; j0 += CB) {
     const int nb = n - j0 < CB ? n - j0 : CB;
     const int rem = n - j0 - nb;
-    const int pg = rem > 0 ? (rem + CB - 1) / CB : 1;
-    double *W = w.dinv + (size_t)(j0 / CB) * CB * CB;
-    k_chol_panel<<<pg, PT, 0, st>>>(w.S, n, j0, nb, w.info, w.dblk, W, w.p, w.w);
+    k_chol_panel<<<1 + (rem + CB - 1) / CB, PT, 0, st>>>(w.S, n, j0, nb, w.info, w.dblk, w.dinv, w.p,
+                                                         w.w);
     if (rem > 0) {
       const int nt = (rem + 31) / 32, tiles = nt * (nt + 1) / 2;
-      k_syrk_trailing<<<tiles + (rem + 255) / 256, 256, 0, st>>>(w.S, n, j0, nb, pg > 1, w.dblk,
-                                                                 tiles, w.p, w.w);
+      k_syrk_trailing<<<tiles + (rem + 255) / 256, 256, 0, st>>>(w.S, n, j0, nb, w.dblk, tiles, w.p, w.w);
     }
   }
   for (int p0 = ((n - 1) / CB) * CB; p0 >= 0; p0 -= CB) {
     const int grid = p0 > 0 ? (p0 + SV_COLS - 1) / SV_COLS : 1;
-    k_trsv_back<<<grid, SV_COLS, 0, st>>>(w.S, n, p0, w.dinv + (size_t)(p0 / CB) * CB * CB, w.w, w.x);
+    k_trsv_back<<<grid, SV_COLS, 0, st>>>(w.S, n, p0, w.dinv, w.w, w.x);
   }
 }
 
