@@ -171,8 +171,8 @@ typedef struct {
   int32_t s_kernel;              /* kernel that built the dense S~: VMC_S_KERNEL_* */
 } vmc_sr_report;
 
-/* vmc_sr_report.s_kernel: no dense S~ (SR-CG product); FP64 SIMT product
- * (plain form); persistent TMA-fed tcgen05 kernel (mixed form); one CTA per
+/* vmc_sr_report.s_kernel: no dense S~ (SR-CG product); product to FP64 accuracy
+ * (plain form, in exact 8-bit digits); persistent TMA-fed tcgen05 kernel (mixed form); one CTA per
  * tile tcgen05 kernel with cp.async staging (mixed form, used when the
  * driver's tensor-map encoder is unavailable or VMC_TC_KERNEL=tiles is set). */
 enum { VMC_S_KERNEL_NONE = 0, VMC_S_KERNEL_FP64 = 1, VMC_S_KERNEL_TMA = 2,

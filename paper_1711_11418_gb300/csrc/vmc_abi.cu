@@ -65,6 +65,10 @@ struct vmc_ctx {
   static constexpr int NPOOL = 8;
   cudaStream_t pool[NPOOL] = {};
   cudaEvent_t fork_ev = nullptr, join_ev[NPOOL] = {};
+  // plain form: workspace of the overlap matrix's digits, one per solver stream
+  // (slot 0 also for the context's stream), shared by the systems of a batch
+  unsigned char *digits[NPOOL] = {};
+  size_t digits_bytes[NPOOL] = {}, digits_asked[NPOOL] = {};
   size_t smem_cap = 0;        // dynamic shared-memory limit set on the sweep kernels
   size_t smem_proj = 0;       // projected sweep kernel (vmc_set_projection)
   size_t smem_build = 0;      // from-scratch inverses of the projected state
@@ -95,6 +99,9 @@ void ctx_free(vmc_ctx *c) {
     if (c->join_ev[k]) cudaEventDestroy(c->join_ev[k]);
     c->pool[k] = nullptr;
     c->join_ev[k] = nullptr;
+    if (c->digits[k]) cudaFree(c->digits[k]);
+    c->digits[k] = nullptr;
+    c->digits_bytes[k] = c->digits_asked[k] = 0;
   }
   if (c->fork_ev) cudaEventDestroy(c->fork_ev);
   c->fork_ev = nullptr;
@@ -419,7 +426,30 @@ int ensure_init(vmc_ctx *c, bool redraw_illcond = false) {
   return VMC_OK;
 }
 
-int sr_alloc(vmc_ctx *c, SysHost &s, bool need_S, bool need_ir = false) {
+// At least one chunk of samples' digits in a solver stream's workspace, better a
+// whole slab; a larger one replaces it (cudaFree waits for the kernels that use
+// it).  One per stream, not per system: 64 systems held 64.
+int digits_alloc(vmc_ctx *c, int slot, int rows_cap, int Np) {
+  const size_t least = vmc_sr_digits_min_bytes(Np), want = vmc_sr_digits_bytes(rows_cap, Np);
+  if (c->digits_bytes[slot] >= least && c->digits_asked[slot] >= want) return VMC_OK;
+  if (c->digits[slot]) cudaFree(c->digits[slot]);
+  c->digits[slot] = nullptr;
+  c->digits_bytes[slot] = 0;
+  const size_t ask = std::max(want, c->digits_asked[slot]);
+  for (size_t b = ask; b >= least; b = b > least ? std::max(least, b / 2) : 0) {
+    if (cudaMalloc((void **)&c->digits[slot], b) == cudaSuccess) {
+      c->digits_bytes[slot] = b;
+      c->digits_asked[slot] = ask;
+      return VMC_OK;
+    }
+    cudaGetLastError();
+    c->digits[slot] = nullptr;
+  }
+  return VMC_ENOMEM;
+}
+
+// slot: the solver stream whose workspace the dense S of this call uses
+int sr_alloc(vmc_ctx *c, SysHost &s, bool need_S, bool need_ir = false, int slot = 0) {
   const int rows_cap = s.W * s.max_samples;
   if (!s.sr_alloc) {
     SrWork &w = s.sr;
@@ -457,18 +487,11 @@ int sr_alloc(vmc_ctx *c, SysHost &s, bool need_S, bool need_ir = false) {
       vmc_tc_tile_list(s.Np, tl.data());
       CK(dupload(c, &s.tc_tiles, tl.data(), tl.size()));
     } else {
-      // the plain form's digits, where there is memory for them (the FP64
-      // kernel builds S otherwise)
-      unsigned char *dg = nullptr;
-      int *em = nullptr;
-      if (dalloc(c, &em, sizeof(int) * (s.Np + 1)) == VMC_OK &&
-          dalloc(c, &dg, vmc_sr_digits_bytes(rows_cap, s.Np)) == VMC_OK) {
-        s.sr.digits = dg;
-        s.sr.emax = em;
-      }
+      CK(dalloc(c, &s.sr.emax, sizeof(int) * (s.Np + 1)));
     }
     s.S_alloc = true;
   }
+  if (need_S && c->precision == VMC_FP64) CK(digits_alloc(c, slot, rows_cap, s.Np));
   s.sr.Np = s.Np;
   s.sr.rows = s.rows;
   s.sr.ldO = s.ldO;
@@ -487,18 +510,26 @@ int sr_alloc(vmc_ctx *c, SysHost &s, bool need_S, bool need_ir = false) {
   return VMC_OK;
 }
 
-// Dense S~: FP64 SIMT GEMM (plain form) or split-BF16 tensor-core GEMM (mixed).
-// Enqueue the S~ build (no host synchronisation; the tensor-core path's
-// status stays on the device).
-int build_S_launch(vmc_ctx *c, SysHost &s, double shift_rel, double shift_abs, cudaStream_t st) {
+// Dense S~ of the plain form, in the workspace of solver stream `slot`.
+int build_S_digits(vmc_ctx *c, SysHost &s, double shift_rel, double shift_abs, cudaStream_t st, int slot) {
+  s.sr.digits = c->digits[slot];
+  s.sr.digits_bytes = c->digits_bytes[slot];
+  CKC(vmc_sr_build_S(s.sr, shift_rel, shift_abs, st, &c->n_launch));
+  s.s_kernel = VMC_S_KERNEL_FP64;
+  return VMC_OK;
+}
+
+// Dense S~: exact 8-bit digit products (plain form) or split-BF16 products
+// (mixed), both on the tensor cores.  Enqueue the S~ build on the solver stream
+// `slot` (no host synchronisation; the mixed path's status stays on the device).
+int build_S_launch(vmc_ctx *c, SysHost &s, double shift_rel, double shift_abs, cudaStream_t st, int slot) {
   if (c->precision == VMC_MIXED) {
     const cudaError_t e = vmc_sr_build_S_tc(s.sr, s.tc_hi, s.tc_lo, s.tc_status, shift_rel,
                                             shift_abs, s.tc_tiles, st, &c->n_launch, &s.s_kernel);
     s.sr.stall = 0;   // the test hook is armed for one build
     CKC(e);
   } else {
-    CKC(vmc_sr_build_S(s.sr, shift_rel, shift_abs, st, &c->n_launch));
-    s.s_kernel = VMC_S_KERNEL_FP64;
+    CK(build_S_digits(c, s, shift_rel, shift_abs, st, slot));
   }
   return VMC_OK;
 }
@@ -517,9 +548,7 @@ int build_S(vmc_ctx *c, SysHost &s, double shift_rel, double shift_abs) {
     if (bad) return VMC_ETIMEOUT;
     return VMC_OK;
   }
-  CKC(vmc_sr_build_S(s.sr, shift_rel, shift_abs, c->st, &c->n_launch));
-  s.s_kernel = VMC_S_KERNEL_FP64;
-  return VMC_OK;
+  return build_S_digits(c, s, shift_rel, shift_abs, c->st, 0);
 }
 
 // From-scratch inverses of every walker; walkers whose M (or, for a projected
@@ -1190,10 +1219,10 @@ int vmc_sr_step_all(vmc_ctx *c, const vmc_sr_opts *o, vmc_sr_report *reps) {
       return VMC_ECUDA;
     }
   }
-  for (auto &s : c->sys) CK(sr_alloc(c, s, true, ir));
+  const int np = std::min(c->n_sys, (int)vmc_ctx::NPOOL);
+  for (int si = 0; si < c->n_sys; ++si) CK(sr_alloc(c, c->sys[si], true, ir, si % np));
   const double eps = o->cg_eps > 0.0 ? o->cg_eps : 1e-12;
   const int kmax = o->cg_kmax > 0 ? std::min(o->cg_kmax, 16) : 8;
-  const int np = std::min(c->n_sys, (int)vmc_ctx::NPOOL);
   // fork: the pool streams wait for everything queued on st so far; join:
   // st waits for the pool.  System si runs on pool[si % np].
   auto fork = [&]() -> int {
@@ -1217,7 +1246,7 @@ int vmc_sr_step_all(vmc_ctx *c, const vmc_sr_opts *o, vmc_sr_report *reps) {
     cudaStream_t st = c->pool[si % np];
     CKC(vmc_sr_means(w, st, &c->n_launch));
     CKC(vmc_sr_build_g(w, false, st, &c->n_launch));
-    CK(build_S_launch(c, s, o->shift_rel, o->shift_abs, st));
+    CK(build_S_launch(c, s, o->shift_rel, o->shift_abs, st, si % np));
     if (c->precision == VMC_MIXED)
       CKC(cudaMemcpyAsync(stg[si].tcstat, s.tc_status, sizeof(int), cudaMemcpyDeviceToHost, st));
     else

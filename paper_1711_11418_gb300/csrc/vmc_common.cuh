@@ -252,16 +252,18 @@ struct SrWork {
   void *ir_graph;
   int ir_iter;
   double ir_eps;
-  unsigned char *digits;       // plain form: a slab of samples as digits (vmc_sr_digits.cu), or null
+  unsigned char *digits;       // plain form: a slab of samples as digits (vmc_sr_digits.cu)
+  size_t digits_bytes;
   int *emax;                   // [Np] exponents of the centred columns, [1] some are not finite
   int stall;                   // test hook: CTA 0 of the next tensor-core S build waits on a
                                // barrier nothing arrives on (then no copy or MMA is issued)
 };
 int vmc_colreduce_parts(int rows, int Np);
 size_t vmc_sr_digits_bytes(int rows, int Np);
-cudaError_t vmc_sr_syrk_digits(const SrWork &w, unsigned char *digits, int *emax, cudaStream_t st,
-                               long long *nl);
+size_t vmc_sr_digits_min_bytes(int Np);
+cudaError_t vmc_sr_syrk_digits(const SrWork &w, cudaStream_t st, long long *nl);
 cudaError_t vmc_sr_means(const SrWork &w, cudaStream_t st, long long *nl);
+// dense S~ of the plain form
 cudaError_t vmc_sr_build_S(const SrWork &w, double shift_rel, double shift_abs,
                            cudaStream_t st, long long *nl);
 // the force g and, with diag, the diagonal of S in the same pass

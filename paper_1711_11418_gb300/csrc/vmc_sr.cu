@@ -161,113 +161,6 @@ __global__ void k_mean_vec(const double *v, int n, double *out) {
   if (threadIdx.x == 0) out[0] = red[0] / n;
 }
 
-// S = (1/rows) (O - o)^T (O - o): 64x64 output tiles of the upper triangle,
-// split over row chunks (atomic accumulation into S, which starts at zero).
-constexpr int ST = 64, SKK = 16;
-template <typename TO>
-__global__ void __launch_bounds__(256) k_syrk(const TO *O, int ldO, int rows, int Np,
-                                              const double *obar, double scale, int rows_per_split,
-                                              double *S) {
-  // map blockIdx.x to an upper-triangular tile pair (bi <= bj)
-  int t = blockIdx.x, bi = 0;
-  const int nt = (Np + ST - 1) / ST;
-  while (t >= nt - bi) {
-    t -= nt - bi;
-    ++bi;
-  }
-  const int bj = bi + t;
-  const int r0 = blockIdx.y * rows_per_split;
-  const int r1 = min(rows, r0 + rows_per_split);
-  __shared__ double As[SKK][ST + 1];
-  __shared__ double Bs[SKK][ST + 1];
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  double acc[4][4] = {};
-  for (int rb = r0; rb < r1; rb += SKK) {
-    for (int q = threadIdx.x; q < SKK * ST; q += 256) {
-      const int rr = q / ST, cc = q % ST;
-      const int r = rb + rr;
-      const int ka = bi * ST + cc, kb = bj * ST + cc;
-      As[rr][cc] = (r < r1 && ka < Np) ? ld(O + (size_t)r * ldO + ka) - obar[ka] : 0.0;
-      Bs[rr][cc] = (r < r1 && kb < Np) ? ld(O + (size_t)r * ldO + kb) - obar[kb] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < SKK; ++kk) {
-      double a[4], b[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        a[u] = As[kk][ty + 16 * u];
-        b[u] = Bs[kk][tx + 16 * u];
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] += a[u] * b[v];
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const int i = bi * ST + ty + 16 * u, j = bj * ST + tx + 16 * v;
-      if (i < Np && j < Np && i <= j) {
-        atomicAdd(S + (size_t)i * Np + j, acc[u][v] * scale);
-      }
-    }
-}
-
-// FP32 variant for the mixed form: FP32 products and FP32 accumulation over
-// at most 1024 rows per split, FP64 accumulation across splits.
-__global__ void __launch_bounds__(256) k_syrk32(const float *O, int ldO, int rows, int Np,
-                                                const double *obar, double scale,
-                                                int rows_per_split, double *S) {
-  int t = blockIdx.x, bi = 0;
-  const int nt = (Np + ST - 1) / ST;
-  while (t >= nt - bi) {
-    t -= nt - bi;
-    ++bi;
-  }
-  const int bj = bi + t;
-  const int r0 = blockIdx.y * rows_per_split;
-  const int r1 = min(rows, r0 + rows_per_split);
-  __shared__ float As[SKK][ST + 1];
-  __shared__ float Bs[SKK][ST + 1];
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  float acc[4][4] = {};
-  for (int rb = r0; rb < r1; rb += SKK) {
-    for (int q = threadIdx.x; q < SKK * ST; q += 256) {
-      const int rr = q / ST, cc = q % ST;
-      const int r = rb + rr;
-      const int ka = bi * ST + cc, kb = bj * ST + cc;
-      As[rr][cc] = (r < r1 && ka < Np) ? (float)((double)O[(size_t)r * ldO + ka] - obar[ka]) : 0.f;
-      Bs[rr][cc] = (r < r1 && kb < Np) ? (float)((double)O[(size_t)r * ldO + kb] - obar[kb]) : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < SKK; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        a[u] = As[kk][ty + 16 * u];
-        b[u] = Bs[kk][tx + 16 * u];
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const int i = bi * ST + ty + 16 * u, j = bj * ST + tx + 16 * v;
-      if (i < Np && j < Np && i <= j) atomicAdd(S + (size_t)i * Np + j, (double)acc[u][v] * scale);
-    }
-}
-
 // Mirror the upper triangle and apply the diagonal shift.
 __global__ void k_mirror_shift(double *S, int Np, double shift_rel, double shift_abs) {
   const size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
@@ -647,35 +540,10 @@ cudaError_t vmc_sr_build_S(const SrWork &w, double shift_rel, double shift_abs, 
                            long long *nl) {
   cudaError_t e = cudaMemsetAsync(w.S, 0, sizeof(double) * (size_t)w.Np * w.Np, st);
   if (e) return e;
+  if ((e = vmc_sr_syrk_digits(w, st, nl))) return e;
   const size_t n2 = (size_t)w.Np * w.Np;
-  if (w.digits) {
-    if ((e = vmc_sr_syrk_digits(w, w.digits, w.emax, st, nl))) return e;
-    k_mirror_shift<<<(unsigned)((n2 + 255) / 256), 256, 0, st>>>(w.S, w.Np, shift_rel, shift_abs);
-    ++*nl;
-    return cudaGetLastError();
-  }
-  const int nt = (w.Np + ST - 1) / ST;
-  const int ntiles = nt * (nt + 1) / 2;
-  int dev = 0, nsm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  int splits = (4 * nsm + ntiles - 1) / ntiles;
-  const int max_splits = (w.rows + 255) / 256;
-  if (splits > max_splits) splits = max_splits;
-  if (w.precision != 0 && splits < (w.rows + 1023) / 1024) splits = (w.rows + 1023) / 1024;
-  if (splits < 1) splits = 1;
-  int rps = (w.rows + splits - 1) / splits;
-  rps = (rps + SKK - 1) / SKK * SKK;
-  splits = (w.rows + rps - 1) / rps;
-  dim3 grid(ntiles, splits);
-  if (w.precision == 0)
-    k_syrk<double><<<grid, 256, 0, st>>>((const double *)w.O, w.ldO, w.rows, w.Np, w.obar,
-                                         1.0 / w.rows, rps, w.S);
-  else
-    k_syrk32<<<grid, 256, 0, st>>>((const float *)w.O, w.ldO, w.rows, w.Np, w.obar,
-                                   1.0 / w.rows, rps, w.S);
   k_mirror_shift<<<(unsigned)((n2 + 255) / 256), 256, 0, st>>>(w.S, w.Np, shift_rel, shift_abs);
-  *nl += 2;
+  ++*nl;
   return cudaGetLastError();
 }
 

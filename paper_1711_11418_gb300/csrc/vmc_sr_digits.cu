@@ -217,28 +217,29 @@ __global__ void __launch_bounds__(256) k_syrk_nonfinite(const double *O, int ldO
   }
 }
 
-// Digit blocks of 16 samples per slab: at most 1 GiB of digits.
-constexpr size_t SLAB_BYTES = 1ull << 30;
+// A slab of samples has at most 256 MiB of digits (17536 samples at 1069
+// parameters), and at least KC samples.
+constexpr size_t SLAB_BYTES = 256ull << 20;
 int pad_blocks(int Np) { return (Np + TS - 1) / TS * (TS / 16); }
-int slab_blocks(int rows, int Np) {
-  const int all = (rows + KC - 1) / KC * (KC / 16);
-  const size_t per = (size_t)NDIG * pad_blocks(Np) * BLK;
-  const size_t most = SLAB_BYTES / per / (KC / 16) * (KC / 16);
-  const size_t kb = most < (size_t)(KC / 16) ? KC / 16 : most;
-  return (size_t)all < kb ? all : (int)kb;
-}
+// bytes of KC samples' digits
+size_t chunk_bytes(int Np) { return (size_t)NDIG * pad_blocks(Np) * BLK * (KC / 16); }
 
 }  // namespace
 
+size_t vmc_sr_digits_min_bytes(int Np) { return chunk_bytes(Np); }
 size_t vmc_sr_digits_bytes(int rows, int Np) {
-  return (size_t)NDIG * pad_blocks(Np) * slab_blocks(rows, Np) * BLK;
+  const size_t all = (size_t)(rows + KC - 1) / KC, most = SLAB_BYTES / chunk_bytes(Np);
+  return chunk_bytes(Np) * (all < most ? all : most > 1 ? most : 1);
 }
 
 // S (upper triangle; zeroed by the caller) += (1/rows) (O - o)^T (O - o) of the
-// FP64 samples; digits: vmc_sr_digits_bytes(rows, Np), emax: Np + 1 ints.
-cudaError_t vmc_sr_syrk_digits(const SrWork &w, unsigned char *digits, int *emax, cudaStream_t st,
-                               long long *nl) {
+// FP64 samples.  w.digits has w.digits_bytes, from vmc_sr_digits_min_bytes(Np)
+// to vmc_sr_digits_bytes(rows, Np), which decide the samples of a slab; w.emax:
+// Np + 1 ints.
+cudaError_t vmc_sr_syrk_digits(const SrWork &w, cudaStream_t st, long long *nl) {
   const double *O = (const double *)w.O;
+  unsigned char *digits = w.digits;
+  int *emax = w.emax;
   cudaError_t e = cudaMemsetAsync(emax, 0, sizeof(int) * (w.Np + 1), st);
   if (e) return e;
   int dev = 0, nsm = 0;
@@ -253,7 +254,9 @@ cudaError_t vmc_sr_syrk_digits(const SrWork &w, unsigned char *digits, int *emax
   if ((e = cudaFuncSetAttribute(k_syrk_dig, cudaFuncAttributeMaxDynamicSharedMemorySize, ST * STAGE)))
     return e;
   const int npb = pad_blocks(w.Np), nt = npb / (TS / 16), ntiles = nt * (nt + 1) / 2;
-  const int slab = slab_blocks(w.rows, w.Np);
+  const size_t all = (size_t)(w.rows + KC - 1) / KC, have = w.digits_bytes / chunk_bytes(w.Np);
+  const int slab = (int)(all < have ? all : have) * (KC / 16);
+  if (slab < 1) return cudaErrorInvalidValue;
   for (int row0 = 0; row0 < w.rows; row0 += slab * 16) {
     const int left = (w.rows - row0 + KC - 1) / KC * (KC / 16);
     const int kb_n = left < slab ? left : slab;
