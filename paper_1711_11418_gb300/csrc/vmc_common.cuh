@@ -132,6 +132,18 @@ inline cudaError_t vmc_smem_limit(const void *kernel, size_t need) {
                               optin - (int)at.sharedSizeBytes);
 }
 
+// 1 / x by two Newton steps from the hardware's 20-bit approximation, the last
+// one a single rounding of a number off by 2^-80: within 0.5 ulp (1 + 2^-20).
+// Very large and small x, infinities and NaNs by the division.
+__device__ __forceinline__ double vmc_recip(double x) {
+  const int e = (int)(((unsigned)__double2hiint(x) >> 20) & 0x7ffu);
+  if (e < 64 || e > 1982) return 1.0 / x;
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  y = fma(fma(-x, y, 1.0), y, y);
+  return fma(fma(-x, y, 1.0), y, y);
+}
+
 // ---- launch wrappers (defined in vmc_walker.cu / vmc_sr.cu) ----
 // All return cudaError_t from the launch; they count launches in *n_launch.
 cudaError_t vmc_launch_expand(const SysDev *h_sys, cudaStream_t st, long long *n_launch);

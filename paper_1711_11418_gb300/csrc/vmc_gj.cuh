@@ -102,17 +102,6 @@ __device__ __forceinline__ long long gj_combine(const float (&a)[8][4], int q) {
   return (long long)p0 * 4294967296ll + (long long)p1 * 65536ll + (long long)p2;
 }
 
-// 1 / x by Newton's iteration from the hardware's 20-bit approximation; very
-// large and small x by the division.
-__device__ __forceinline__ double gj_recip(double x) {
-  const int e = vmc_dig::expo(x);
-  if (e < 64 || e > 1982) return 1.0 / x;
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  y = fma(fma(-x, y, 1.0), y, y);
-  return fma(fma(-x, y, 1.0), y, y);
-}
-
 // GB elimination steps on the panel of columns k0 .. k0 + GB - 1; threads
 // tid < 32 ceil(Npad / 32), row tid each.  `mine` is the step of which this
 // thread's row is the pivot (-1: none yet), `piv` that pivot.  Per step each
@@ -144,7 +133,7 @@ __device__ __forceinline__ void gj_panel(double *A, int ld, int Npad, int k0, in
     if (bal ? lane == __ffs(bal) - 1 : lane == 0) {
       g.ckey[buf][warp] = bal ? ((unsigned long long)mh << 32) | ml : 0ull;
       g.crow[buf][warp] = tid;
-      g.cinv[buf][warp] = gj_recip(r[k]);
+      g.cinv[buf][warp] = vmc_recip(r[k]);
 #pragma unroll
       for (int j = 0; j < GB; j += 2)
         *reinterpret_cast<double2 *>(&g.cand[buf][warp][j]) = make_double2(r[j], r[j + 1]);

@@ -185,17 +185,6 @@ __global__ void k_mirror_shift(double *S, int Np, double shift_rel, double shift
 constexpr int CB = 32;
 constexpr int PT = 128;    // threads of k_chol_panel
 
-// 1 / x by Newton's iteration from the hardware's 20-bit approximation; very
-// large and small x by the division.
-__device__ __forceinline__ double fast_recip(double x) {
-  const int e = (int)(((unsigned)__double2hiint(x) >> 20) & 0x7ffu);
-  if (e < 64 || e > 1982) return 1.0 / x;
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  y = fma(fma(-x, y, 1.0), y, y);
-  return fma(fma(-x, y, 1.0), y, y);
-}
-
 // Panel step.  Every CTA factors the nb x nb diagonal block redundantly, lane =
 // row, warp w the columns w, w + 4, ...: elimination without square roots
 // (A = L1 D L1^T, L1 unit), L_jj = L1 D^1/2.  All CTAs but the last then solve
@@ -239,7 +228,7 @@ __global__ void __launch_bounds__(PT) k_chol_panel(double *A, int n, int j0, int
         if (r == 0 && !bad_sh) bad_sh = k + 1;
         piv = 1.0;
       }
-      const double ip = fast_recip(piv);
+      const double ip = vmc_recip(piv);
       const double m = r > k ? a[k >> 2] * ip : 0.0;
       acol[b][r] = a[k >> 2];
       mcol[b][r] = m;
