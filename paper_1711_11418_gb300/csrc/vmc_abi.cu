@@ -562,18 +562,19 @@ int init_with_redraw(vmc_ctx *c, uint64_t state) {
     for (SysHost &s : c->sys) {
       std::vector<int> st(s.W);
       std::vector<int32_t> ele((size_t)s.W * s.Ne);
-      if (cudaMemcpy(st.data(), s.dev.status, sizeof(int) * s.W, cudaMemcpyDeviceToHost) ||
-          cudaMemcpy(ele.data(), s.dev.ele, sizeof(int32_t) * ele.size(), cudaMemcpyDeviceToHost))
-        return VMC_ECUDA;
+      // on the context's stream: a copy on the default stream may still be on its
+      // way when it returns, and another stream does not wait for it
+      CKC(cudaMemcpyAsync(st.data(), s.dev.status, sizeof(int) * s.W, cudaMemcpyDeviceToHost, c->st));
+      CKC(cudaMemcpyAsync(ele.data(), s.dev.ele, sizeof(int32_t) * ele.size(), cudaMemcpyDeviceToHost, c->st));
+      CKC(cudaStreamSynchronize(c->st));
       for (int w = 0; w < s.W; ++w)
         if (st[w] & (VMC_ST_SINGULAR | VMC_ST_ILLCOND))
           random_placement(s.Ns, s.Ne, s.dev.local_spin != 0,
                            s.lsite.empty() ? nullptr : s.lsite.data(), state,
                            ele.data() + (size_t)w * s.Ne);
-      std::vector<int> zero(s.W, 0);
-      if (cudaMemcpy(s.dev.ele, ele.data(), sizeof(int32_t) * ele.size(), cudaMemcpyHostToDevice) ||
-          cudaMemcpy(s.dev.status, zero.data(), sizeof(int) * s.W, cudaMemcpyHostToDevice))
-        return VMC_ECUDA;
+      CKC(cudaMemcpyAsync(s.dev.ele, ele.data(), sizeof(int32_t) * ele.size(), cudaMemcpyHostToDevice, c->st));
+      CKC(cudaMemsetAsync(s.dev.status, 0, sizeof(int) * s.W, c->st));
+      CKC(cudaStreamSynchronize(c->st));
     }
   }
 }

@@ -79,3 +79,25 @@ def test_power_lanczos_from_two_threads():
     assert not errors
     for k in range(2):
         assert all(np.array_equal(x, out[k][0]) for x in out[k])
+
+
+@pytest.mark.parametrize("precision", [vmc.FP64, vmc.MIXED])
+def test_placements_redrawn_on_the_contexts_stream(precision):
+    """A third of the random placements are singular and drawn again, on a stream
+    that does not wait for the default one: inverses and sites belong together."""
+    import torch
+
+    p = I.make_problem("redraw", I.square(8, 8), 6, sub=(1, 1), f_full=True, f_init="none", noise=0.0)
+    f = np.random.default_rng(1).standard_normal((p.Ns, p.Ns))
+    f[:8] = 0.0
+    params = p.params.copy()
+    params[p.n_g + p.n_v:] = f.reshape(-1)
+    W = 3000
+    st = torch.cuda.Stream()
+    with vmc.Context(p.copy_with(params=params), W, seed=9, precision=precision, stream=st.cuda_stream) as ctx:
+        ele, _ = ctx.get_configs()
+        assert ele[:, :3].min() >= 8
+        for w in range(0, W, 50):
+            X = ctx.get_inverse(w)[0]
+            M = f[np.ix_(ele[w, :3], ele[w, 3:])]
+            assert np.abs(X @ M - np.eye(3)).max() <= 1e-12 * np.linalg.cond(M)
