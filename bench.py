@@ -810,9 +810,11 @@ def run_ours(args):
     # device time in the timed region is reported as `roofline`.
     #  sweep + measurement (k_sample<float>): FP32 FLOPs from its counters per
     #    launch / launch time, against the FP32 ALU peak; its HBM fraction beside;
-    #  from-scratch inverses (k_init<float>): 2 N^3 FP64 FLOPs per inverse
-    #    (every walker after each SR step, plus in-sweep recomputes) / time,
-    #    against the FP64 peak.
+    #  from-scratch inverses (k_init<float>): what the elimination by panels of
+    #    GB = 16 columns leaves the FP64 pipe (Npad^2 GB multiply-adds in the
+    #    panels, Npad^2 additions per panel in the updates, whose products run in
+    #    8-bit digits on the tensor cores) per inverse (every walker after each SR
+    #    step, plus in-sweep recomputes) / time, against the FP64 peak.
     hbm, hbm_src = hbm_peak_gbs()
     scale = args.walkers / 4096.0
     f32, f64rec = flops_of(mixed["stats"], N, "mixed")
@@ -849,16 +851,22 @@ def run_ours(args):
                                "timed after the timed region on the same context"}
     init_ms, _ = mixed["kt"]["init"]
     n_inv = args.steps * args.walkers + mixed["stats"]["n_recomputes"]
-    ach_init = 2.0 * N ** 3 * n_inv / max(init_ms * 1e-3, 1e-12) / 1e12
+    npad, gb = -(-N // 16) * 16, 16
+    fp64_ops = npad * npad * (2.0 * gb + npad / gb)
+    init_s = max(init_ms * 1e-3, 1e-12)
+    ach_init = fp64_ops * n_inv / init_s / 1e12
     roof_init = {"bound": "alu", "achieved": ach_init, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                  "frac": ach_init / FP64_PEAK_TFLOPS, "traffic": TRAFFIC_INIT_4096 * scale,
                  "traffic_launch": "the full rebuild of all walkers after an SR step",
                  "kernel": "k_init<float> (FP64 from-scratch inverses)",
                  "ms_in_timed_region": init_ms,
+                 "fp64_ops_per_inverse": fp64_ops,
+                 "ops_rule": "Npad^2 (2 x 16 + Npad / 16): the panels' multiply-adds and the updates' "
+                             "additions; the updates' products run in exact 8-bit digits on the "
+                             "tensor cores",
+                 "equivalent_2n3_tflops": 2.0 * N ** 3 * n_inv / init_s / 1e12,
                  "peak_source": "derived: 152 SMs x 2 FP64 FMA units x 2 x 2070 MHz "
-                                "(a DFMA throughput loop measured 1.198 TFLOP/s); the rank-16 "
-                                "updates run in exact 8-bit digits on the tensor cores, so the "
-                                "rate of 2 N^3 per inverse can exceed it"}
+                                "(a DFMA throughput loop measured 1.198 TFLOP/s)"}
     roof, roof2 = (roof_init, roof_sweep) if init_ms > sweep_ms else (roof_sweep, roof_init)
     roof["measured_gemm_tflops"] = peaks
     pair_corr = None

@@ -380,9 +380,6 @@ int periodic_rebuild(vmc_ctx *c) {
   return VMC_OK;
 }
 
-// Every inverse current before it is read: the full rebuild after a parameter
-// or configuration change, else the periodic rebuild the last vmc_sample left
-// pending (a full rebuild makes that one moot).
 // Every walker's status bits, all systems' in one copy: a wait and a copy per
 // system were 8 us each (64 systems: 0.5 ms a call).
 int status_bits(vmc_ctx *c, int *bad) {
@@ -395,6 +392,9 @@ int status_bits(vmc_ctx *c, int *bad) {
   return VMC_OK;
 }
 
+// Every inverse current before it is read: the full rebuild after a parameter
+// or configuration change, else the periodic rebuild the last vmc_sample left
+// pending (a full rebuild makes that one moot).
 int ensure_init(vmc_ctx *c, bool redraw_illcond = false) {
   bool any = false;
   for (auto &s : c->sys) any |= s.dirty;
@@ -860,6 +860,10 @@ int create_impl(vmc_ctx **out, int n_sys, const vmc_model *models, const int32_t
   // Plain form: the O rows are accumulated in their global rows where that lets
   // a second CTA onto the SM (FP64 M^-1 of N = 112 with 1069 parameters: 117
   // against 110 KB a walker; 1024 walkers, a sweep and a measurement 8.4 -> 6.1 ms).
+  // Batches of proposals and delayed updates need the space again, and few walkers
+  // have no use for the second CTA; the global rows cost nothing there either (b =
+  // 4: 8.56 ms, 8.65 in shared memory; delay 8: 7.11 and 7.21; 100 walkers: 1.18
+  // and 1.17).
   if (c->precision == VMC_FP64 && vmc_sample_occupancy(0, smem64) < 2 &&
       vmc_sample_occupancy(0, smem64g) >= 2)
     for (SysHost &s : c->sys) s.dev.acc_len = 0;

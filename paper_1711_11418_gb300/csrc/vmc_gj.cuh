@@ -28,9 +28,9 @@
 //
 // What bounds it: the FP64 pipe (2 multiply-adds per clock and SM), which has
 // the panels' N^2 GB multiply-adds and the update's N^3 / GB additions left
-// of N^3, and the pivot chain of the panels.  4096 walkers, N = 112: 5.1 ms
-// against 13.65 step by step; N = 128: 9.0 against 26.7; N = 64: 1.8 against
-// 3.2.  mma.sync and not tcgen05: a tile's products are consumed at once
+// of N^3, and the pivot chain of the panels.  4096 walkers, mixed form, with the
+// walkers close to singular done again: N = 112 5.9 ms against 13.65 step by
+// step; N = 128 9.5 against 26.7; N = 64 2.0 against 3.2.  mma.sync and not tcgen05: a tile's products are consumed at once
 // by the warp that made them, eight 112 x 112 accumulators do not fit tensor
 // memory, and two walkers share an SM so that one's panel chain runs under
 // the other's update.
@@ -369,18 +369,18 @@ __device__ __forceinline__ double gj_inverse_at(const double *A, int N, int k, i
 // ---------------------------------------------------------------------------
 // The elimination step by step, every multiply-add in FP64.  The blocked form
 // above differs from it in the last bits (about 1e-14 of the inverse, at no
-// larger error).  It takes the matrices close to singular; and two users of the
-// inverse turn last bits into visible
-// differences of a trajectory and keep this form: the mixed form's projected
+// larger error).  It takes the matrices close to singular, of the plain and the
+// projected state alike (gj_invert_guarded); and two users of the inverse turn
+// last bits into visible differences of a trajectory and keep this form: the mixed form's projected
 // state, whose FP32 inverses have no low words and whose ratios are sums over
 // the operations that cancel, and the mixed form of models with exchange
 // terms, whose SR-CG steps stop before convergence and follow the last bits
 // of the samples (a relative change of 1e-9 in E moves the step by up to 5 %).
 // Threads: 128, or 256 where one CTA fills an SM's shared memory (N > 112).
 // The N^3 multiply-adds keep the FP64 pipe 67 % busy at N = 112, two CTAs per
-// SM; a form with the matrix in registers (16 x 16 threads, one CTA per SM)
-// was slower there, 645 against 465 ms for 608 x 256 inverses: nothing runs
-// under its chain of pivots.
+// SM (608 x 256 inverses: 480 ms); a form with the matrix in registers (16 x 16
+// threads, one CTA per SM) was slower there, 645 ms: nothing runs under its chain
+// of pivots.
 // In place on an N x N row-major matrix (row stride lda) in shared or global
 // memory.  Two barriers per elimination step:
 //   (P, B) two warps take the pivot of column k from the per-warp
@@ -424,7 +424,8 @@ struct GJSteps {
 // correlations differ from those of the step-by-step inverses by up to 0.8 of
 // their size with the blocked form alone, by 2e-5 with 3000 here (5e-7 with
 // 1000); k_init takes 5.1, 5.9 and 6.2 ms.  About one random placement in 270
-// is above.
+// is above.  (Set on placements at N = 112; the bound itself does not depend on
+// N.)
 constexpr double GJ_BLOCKED_COND = 3e3;
 // Where the second elimination keeps GJSteps: in the staged digits' space,
 // behind the part that its longer rows (odd stride) take.

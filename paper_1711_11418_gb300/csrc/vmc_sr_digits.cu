@@ -21,9 +21,10 @@
 // FP64; 4 clocks per m16n8k16 and SM).  16384 x 1069: 2.2 ms, and 0.11 ms for
 // the digits, against 21.2 ms on the FP64 pipe (15.6 ms at its full rate).
 // Error against quad precision, relative to sqrt(S_kk S_mm): 2.0e-17 rms for
-// normal columns (FP64 pipe 2.1e-17), largest 5.2e-16 with heavy tails (6.0e-16).  mma.sync and not tcgen05: eight accumulators of a
-// 128 x 128 tile are twice the tensor memory, and every 128 samples they would
-// all be read back.
+// normal columns (FP64 pipe 2.1e-17), largest
+// 5.2e-16 with heavy tails (6.0e-16).  mma.sync and not tcgen05: the eight FP32
+// accumulators of a 128 x 64 tile fill tensor memory, and every 128 samples they
+// would all be read back; that kernel was not built.
 #include "vmc_common.cuh"
 #include "vmc_digits.cuh"
 

@@ -2552,9 +2552,12 @@ extern "C" void vmc_init_plan(int precision, int df, int exchange, int n_sys, co
                               const int *Ns, int n_work, int n_sm, InitPlan *plan) {
   int n_max = 1;
   for (int s = 0; s < n_sys; ++s) n_max = N[s] > n_max ? N[s] : n_max;
-  // a walker per SM or fewer: one walker's time is the launch's, and up to N = 48
-  // it is shorter step by step (125 walkers at N = 36, four samples with rebuilds
-  // 1218 -> 1159 us; the gradient of 110 at N = 38 316 -> 308)
+  // a walker per SM or fewer: one walker's time is the launch's, and a walker close
+  // to singular (about one in 270) makes it panels and steps.  FP64, N = 25, 32, 36,
+  // 40, 44, 48: 66, 75, 95, 110, 119, 137 us step by step; 66, 66, 101, 100, 99, 100
+  // by panels, 137 to 235 with such a walker.  So from about 64 walkers on the steps
+  // are shorter on average up to N = 48 (125 walkers at N = 36, four samples with
+  // rebuilds 1218 -> 1159 us); below, panels would win by a tenth at N >= 44.
   const bool few = n_work <= n_sm && n_max <= 48;
   if (precision != 0 && df) plan->form = VMC_INIT_DF;
   else if ((precision != 0 && exchange) || n_max <= vmc_gj::GJ_STEPS_MAX_N || few) plan->form = VMC_INIT_STEPS;
